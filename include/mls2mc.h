@@ -184,14 +184,13 @@ int smc_set_timing(smc_handle* h, int enable);
  * block size (threads per particle) on n_tune prior draws and keep the fastest for the process
  * (shared by all handles of the same 1/h and precision). chosen [n_levels] receives the block
  * sizes, best_ms [n_levels] the time per launch (either may be NULL). smc_set_block_size forces a
- * block size for a level (T = 0 restores the default: the compact form on 1/32 and 1/64 of the
- * mixed path, the two-CTA form on 1/128, else the first compiled size); T must be one of the
- * compiled sizes. A negative size -T selects the compact form with T threads per particle (mixed
- * precision: -512 at 1/h = 64, -256 at 1/h = 32): several particles per SM, the fine level in five
- * arrays and each coarse level in four, the refinement state in device memory (same results as the
- * size T, bit for bit). At 1/h = 128, -1024 selects the two-CTA form: one particle per cluster of two
- * CTAs of 1024 threads on two SMs, each keeping half of the fine rows on chip with one halo row from
- * the other through distributed shared memory, the coarse levels 1/64 .. 1/2 in both (the same
+ * block size for a level (T = 0 restores the default: -512 and -256 on 1/64 and 1/32 of the mixed
+ * path, the two-CTA form on 1/128, else the first compiled size); T must be one of the
+ * compiled sizes. On 1/64 (512, 1024, -512) and 1/32 (256, 512, -256) of the mixed path every size
+ * names the same register-tiled form (two particles per SM on 1/64, eight on 1/32; the flow cell has one
+ * form per level of its own). At 1/h = 128, -1024 selects the two-CTA form: one particle per cluster of
+ * two CTAs of 1024 threads on two SMs, each keeping half of the fine rows on chip with one halo row
+ * from the other through distributed shared memory, the coarse levels 1/64 .. 1/2 in both (the same
  * algorithm as 1024, which keeps the fine level in device memory; potentials agree to rounding).
  * Batched solves on 1/128 run the two-CTA form where a cluster fits; flow-cell solves the
  * device-memory form. */

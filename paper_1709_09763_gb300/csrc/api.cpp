@@ -37,7 +37,7 @@ static int tuned_block(int N, int precision) {
     return it == g_block.end() ? 0 : it->second;
 }
 
-// T = 0: the default; T < 0: the compact form with -T threads (where compiled)
+// T = 0: the default
 static void set_block(int N, int precision, int T) {
     std::lock_guard<std::mutex> lock(g_tune_mu);
     if (T == 0) g_block.erase({N, precision});
@@ -248,16 +248,15 @@ int Handle::eval_device(int level, int n, const double* theta, double* G, double
         int T = tuned_block(L.N, precision);
         if (T == 0) T = fem_default_block(L.N, precision);
         if (flow_cell) T = 0;   // the flow cell has one (one-block) form per level
-        if (T < 0) {   // compact form: persistent blocks with their refinement state in device memory
-            const int blocks = fem_compact_blocks(L.N, -T);
-            if (blocks <= 0) return fail(SMC_EINVAL, "no compact form with %d threads at 1/h = %d", -T, L.N);
-            const size_t need = (size_t)blocks * fem_compact_ref_floats(L.N, -T);
+        if (fem_tile_form(L.N, precision, flow_cell != 0)) {
+            // register-tiled form: persistent blocks with their refinement state in device memory
+            const size_t need = fem_tile_scratch(L.N);
             if (need > cp_cap) {
                 cudaFree(cp_scratch);
                 cp_scratch = nullptr;
                 cp_cap = 0;
                 cudaError_t ea = cudaMalloc((void**)&cp_scratch, need * sizeof(float));
-                if (ea != cudaSuccess) return fail(SMC_ENOMEM, "compact-form scratch: %s", cudaGetErrorString(ea));
+                if (ea != cudaSuccess) return fail(SMC_ENOMEM, "tile-form scratch: %s", cudaGetErrorString(ea));
                 cp_cap = need;
             }
             if (!big_counter && cudaMalloc((void**)&big_counter, sizeof(int)) != cudaSuccess)
@@ -268,7 +267,7 @@ int Handle::eval_device(int level, int n, const double* theta, double* G, double
                 t.stop = take_event();
                 cudaEventRecord(t.start, st);
             }
-            e = fem_eval_compact_launch(a, -T, cp_scratch, blocks, big_counter, st);
+            e = fem_tile_launch(a, cp_scratch, big_counter, st);
             if (timing) {
                 cudaEventRecord(t.stop, st);
                 timed.push_back(t);

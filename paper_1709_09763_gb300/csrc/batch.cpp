@@ -10,7 +10,6 @@
 
 #include <algorithm>
 #include <cstring>
-#include <cstdlib>
 #include <map>
 #include <string>
 #include <vector>
@@ -39,6 +38,9 @@ int enqueue(Batch* b, const int* level, const int* n, const double* const* theta
         if (G.N >= 128)   // the form single solves default to (two-CTA on 1/128)
             e = fem_eval_large_multi_launch(G.N, G.d_args, G.d_offsets, G.d_item_group, G.total, b->big_scratch,
                                             b->d_counters + g, st);
+        else if (fem_tile_form(G.N, G.precision, false))
+            e = fem_tile_multi_launch(G.N, G.d_args, G.d_offsets, G.d_item_group, G.total, b->big_scratch,
+                                      b->d_counters + g, st);
         else
             e = fem_eval_persistent_launch(G.N, G.precision, G.T, G.d_args, G.d_offsets, G.d_item_group, G.total,
                                            b->d_counters + g, st);
@@ -122,9 +124,7 @@ int smc_batch_eval(smc_batch* bb, const int* level, const int* n, const double* 
                 Batch::Group G;
                 G.N = L.N;
                 G.precision = h->precision;
-                // the persistent form has no compact variant: a compact size -T runs with T threads,
-                // the same arithmetic
-                G.T = std::abs(h->block_size(L.N));
+                G.T = h->block_size(L.N);
                 b->groups.push_back(G);
             }
             Batch::Group& G = b->groups[gidx[key]];
@@ -135,9 +135,8 @@ int smc_batch_eval(smc_batch* bb, const int* level, const int* n, const double* 
             G.total += n[p];
         }
         cudaError_t e = cudaMalloc((void**)&b->d_counters, sizeof(int) * std::max<size_t>(1, b->groups.size()));
-        size_t big_need = 0;   // one scratch for all large groups: they run one after another
-        for (auto& G : b->groups)
-            if (G.N >= 128) big_need = std::max(big_need, fem_large_multi_scratch(G.N));
+        size_t big_need = 0;   // one scratch for all groups: they run one after another
+        for (auto& G : b->groups) big_need = std::max(big_need, fem_multi_scratch(G.N, G.precision));
         if (e == cudaSuccess && big_need) e = cudaMalloc((void**)&b->big_scratch, big_need * sizeof(float));
         for (auto& G : b->groups) {
             if (e == cudaSuccess) e = cudaMalloc((void**)&G.d_args, sizeof(FemArgs) * G.args.size());

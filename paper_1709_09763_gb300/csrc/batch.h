@@ -27,7 +27,7 @@ struct Batch {
     };
     std::vector<Group> groups;
     int* d_counters = nullptr;
-    float* big_scratch = nullptr;    // per-block (per-CTA) scratch of the groups of large levels (1/h >= 128)
+    float* big_scratch = nullptr;    // per-block (per-CTA) scratch of the groups' solves (fem_multi_scratch)
     std::vector<long long> signature;
     cudaGraph_t graph = nullptr;
     cudaGraphExec_t exec = nullptr;

@@ -151,8 +151,7 @@ int multi_eval(Batch* b, const std::vector<EvalReq>& reqs, cudaStream_t st) {
             Handle* h = b->h[q.p];
             const auto k = key(idx[r]);
             if (groups.empty() || groups.back().N != k.first || groups.back().precision != k.second) {
-                // the persistent form has no compact variant: a compact size -T runs with T threads
-                groups.push_back({k.first, k.second, std::abs(h->block_size(k.first)), (int)r, 0, 0, items});
+                groups.push_back({k.first, k.second, h->block_size(k.first), (int)r, 0, 0, items});
             }
             G& g = groups.back();
             FemArgs a = h->fem_args(q.level, q.n, q.theta, nullptr, q.phi, h->smp->iters);
@@ -182,14 +181,13 @@ int multi_eval(Batch* b, const std::vector<EvalReq>& reqs, cudaStream_t st) {
             S->item_cap = (size_t)items;
         }
         size_t big_need = 0;
-        for (const G& g : groups)
-            if (g.N >= 128) big_need = std::max(big_need, fem_large_multi_scratch(g.N));
+        for (const G& g : groups) big_need = std::max(big_need, fem_multi_scratch(g.N, g.precision));
         if (big_need > S->big_cap) {
             cudaFree(S->big_scratch);
             S->big_scratch = nullptr;
             S->big_cap = 0;
             if (cudaMalloc((void**)&S->big_scratch, big_need * sizeof(float)) != cudaSuccess)
-                return bfail(b, SMC_ENOMEM, "batched sampler: large-level scratch");
+                return bfail(b, SMC_ENOMEM, "batched sampler: solve scratch");
             S->big_cap = big_need;
         }
         const int threads = 256, blocks = std::max(1, std::min(1024, (items + threads - 1) / threads));
@@ -202,6 +200,9 @@ int multi_eval(Batch* b, const std::vector<EvalReq>& reqs, cudaStream_t st) {
                 e = fem_eval_large_multi_launch(g.N, S->d_args + g.first, S->d_offsets + g.first,
                                                 S->d_item_group + g.item_base, g.total, S->big_scratch,
                                                 S->d_counters + gi, st);
+            else if (fem_tile_form(g.N, g.precision, false))
+                e = fem_tile_multi_launch(g.N, S->d_args + g.first, S->d_offsets + g.first,
+                                          S->d_item_group + g.item_base, g.total, S->big_scratch, S->d_counters + gi, st);
             else
                 e = fem_eval_persistent_launch(g.N, g.precision, g.T, S->d_args + g.first, S->d_offsets + g.first,
                                                S->d_item_group + g.item_base, g.total, S->d_counters + gi, st);
@@ -248,13 +249,12 @@ int batch_step(Batch* b, smc_stage_info* infos) {
         if (e == cudaSuccess) e = cudaMalloc((void**)&S->d_offsets, sizeof(int) * kMaxTasks);
         if (e == cudaSuccess) e = cudaMalloc((void**)&S->d_counters, sizeof(int) * kMaxTasks);
         if (e == cudaSuccess) e = cudaMallocHost((void**)&S->back, sizeof(BatchSampler::Back) * (size_t)P);
-        // the largest item table and large-level scratch a step can need, allocated now: the update
+        // the largest item table and solve scratch a step can need, allocated now: the update
         // phase is captured into a graph, where nothing may be allocated
         size_t items = 0, big = 0;
         for (Handle* h : b->h) {
             items += (size_t)h->smp->J;
-            for (const Level& L : h->levels)
-                if (L.N >= 128) big = std::max(big, fem_large_multi_scratch(L.N));
+            for (const Level& L : h->levels) big = std::max(big, fem_multi_scratch(L.N, h->precision));
             // the syntheses' buffers at their largest (J particles on the finest level): a buffer that
             // grew inside a captured update would free memory that earlier captured launches use
             if (h->precision == SMC_MIXED) {

@@ -31,9 +31,8 @@
 // vectors e (multigrid correction), res (residual) and rhs (fine level: the CG
 // direction p). The fine-level CG vectors r, d, z, p of a thread's nodes live in
 // registers (every fine node belongs to one thread for the whole solve); the
-// refinement state x, r (double-float pairs) lives in shared memory, or in a per-block
-// slice of device memory in the compact forms (two or four blocks per SM, coarse levels
-// without residual and inverse-diagonal arrays). Level 1/128 is solved by a cluster of two CTAs
+// refinement state x, r (double-float pairs) lives in shared memory. The mixed Dirichlet solve on 1/64
+// and 1/32 has a form of its own (fem_tile.cu). Level 1/128 is solved by a cluster of two CTAs
 // on two SMs, each keeping half of the fine rows on chip (fem_eval_cluster); levels 1/128 (block
 // size 1024, the flow cell) and 1/256 can keep their two finest levels in device memory
 // (fem_eval_global).
@@ -44,6 +43,7 @@
 #include <cstdint>
 #include <vector>
 
+#include "fem_device.h"
 #include "internal.h"
 
 namespace mls2mc {
@@ -69,17 +69,15 @@ struct Lv {
     Real *aE, *aN, *iD, *e, *res, *rhs;   // iD: inverse of the stencil diagonal
 };
 
-// Compact hierarchy (two blocks per SM at 1/64): the top level keeps five arrays (res shares
-// the storage of rhs, which holds the CG direction p: p is dead while the V-cycle runs, its
-// values live in registers), the coarse levels four (aE, aN, e, rhs: no res, and the inverse
-// diagonal is formed from the edge weights where a sweep needs it).
+// Coarse hierarchy of the two-CTA form (levels N/2 .. 2): four arrays a level (aE, aN, e, rhs: no res,
+// and the inverse diagonal is formed from the edge weights where a sweep needs it).
 __host__ __device__ constexpr int coarse_size_cp(int NL) { return NL < 2 ? 0 : 4 * lvl_size(NL) + coarse_size_cp(NL / 2); }
 __host__ __device__ constexpr int coarse_offset_cp(int NL, int NC) {
     return NL == NC ? 0 : 4 * lvl_size(NL) + coarse_offset_cp(NL / 2, NC);
 }
-__host__ __device__ constexpr int arena_size_cp(int N) { return 5 * lvl_size(N) + coarse_size_cp(N / 2); }
 
-template <typename Real, int N, int NL, int CP = 0, bool FC = false>
+// CP: the coarse hierarchy of the two-CTA form (NL < N), from the arena's start
+template <typename Real, int N, int NL, bool CP = false, bool FC = false>
 __device__ __forceinline__ Lv<Real> level_ptrs(Real* arena) {
     if constexpr (FC) {   // ghost row -1 first: each pointer is one row stride into its array
         constexpr int z = lvl_size(NL, true);
@@ -90,15 +88,9 @@ __device__ __forceinline__ Lv<Real> level_ptrs(Real* arena) {
     if constexpr (!CP) {
         Real* b = arena + lvl_offset(N, NL);
         return Lv<Real>{b, b + z, b + 2 * z, b + 3 * z, b + 4 * z, b + 5 * z};
-    } else if constexpr (CP == 2) {   // coarse levels N/2 .. 2 alone, from the arena's start
+    } else {
         static_assert(NL < N, "the two-CTA form keeps its top level apart");
         Real* b = arena + coarse_offset_cp(N / 2, NL);
-        return Lv<Real>{b, b + z, nullptr, b + 2 * z, nullptr, b + 3 * z};
-    } else if constexpr (NL == N) {
-        Real* b = arena;
-        return Lv<Real>{b, b + z, b + 2 * z, b + 3 * z, b + 4 * z, b + 4 * z};
-    } else {
-        Real* b = arena + 5 * lvl_size(N) + coarse_offset_cp(N / 2, NL);
         return Lv<Real>{b, b + z, nullptr, b + 2 * z, nullptr, b + 3 * z};
     }
 }
@@ -113,20 +105,6 @@ __device__ __forceinline__ void load_rhs(const void* t, int n, float& hi, float&
     hi = v.x;
     lo = v.y;
 }
-
-// 1 / x rounded to nearest (the same value as the IEEE division 1 / x)
-__device__ __forceinline__ float recip(float x) { return __frcp_rn(x); }
-__device__ __forceinline__ double recip(double x) { return __drcp_rn(x); }
-// The smoother's inverse diagonals on the coarse levels: the approximate reciprocal of the special
-// function unit (one instruction, relative error below 2^-22) on the FP32 path. They only shape the
-// multigrid preconditioner -- the CG operator and the refinement residual use the edge weights --
-// and the preconditioner stays symmetric because every sweep uses the same value at a node.
-__device__ __forceinline__ float recip_coarse(float x) {
-    float r;
-    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
-    return r;
-}
-__device__ __forceinline__ double recip_coarse(double x) { return __drcp_rn(x); }
 
 // inverse stencil diagonal at interior node n: stored, or formed from the four edge weights
 // (the same expression and order as where it is stored)
@@ -170,24 +148,6 @@ __device__ __forceinline__ void block_sum(Acc& a, double* buf_raw) {
 #pragma unroll
     for (int i = 0; i < T / 32; ++i) s += buf[i];
     a = s;
-}
-
-// ---- error-free transformations (Knuth TwoSum, Dekker), double-float accumulation ----
-template <typename Real>
-__device__ __forceinline__ void two_sum(Real a, Real b, Real& s, Real& e) {
-    s = a + b;
-    const Real bb = s - a;
-    e = (a - (s - bb)) + (b - bb);
-}
-
-// (ah, al) += (bh, bl), result renormalised so that |al| <= ulp(ah)/2
-template <typename Real>
-__device__ __forceinline__ void df_add(Real& ah, Real& al, Real bh, Real bl) {
-    Real s, e;
-    two_sum(ah, bh, s, e);
-    e += al + bl;
-    ah = s + e;
-    al = e - (ah - s);
 }
 
 // ---- red/black enumeration -----------------------------------------------------------------
@@ -270,7 +230,7 @@ __device__ __forceinline__ void restrict_gather(const Real* res, const Lv<Real>&
 
 // zero the boundary rings of e, res, rhs on every level from NL down (interior values are always
 // written before they are read; the rings must read as zero)
-template <typename Real, int N, int NL, int T, int CP = 0, bool FC = false>
+template <typename Real, int N, int NL, int T, bool CP = false, bool FC = false>
 __device__ __forceinline__ void zero_rings(Real* arena) {
     constexpr int S = fem_row_stride(NL);
     const Lv<Real> L = level_ptrs<Real, N, NL, CP, FC>(arena);
@@ -419,7 +379,7 @@ __device__ __forceinline__ void phase_sync() {
 // V(1,1) cycle on a coarse level: reads L.rhs, writes L.e. Levels with at most 4 cells per side
 // (<= 9 unknowns) run inside warp 0 only (T = 32, warp barriers); the caller's next block
 // barrier publishes the result.
-template <typename Real, int N, int NL, int T, bool WARP = false, int CP = 0, bool FC = false>
+template <typename Real, int N, int NL, int T, bool WARP = false, bool CP = false, bool FC = false>
 __device__ void vcycle_coarse(Real* arena, const Real* dinv) {
     if constexpr (NL == direct_level<Real, FC>(N)) {
         dense_solve<Real, NL, T, FC>(level_ptrs<Real, N, NL, CP, FC>(arena), dinv);
@@ -519,16 +479,16 @@ __device__ void setup_levels(Real* arena, Real* stage, bool ping) {
     }
 }
 
-// compact hierarchy: coefficients of coarse level NL from kappa in kin, coarser kappa into kout,
-// then recurse with the buffers swapped (no stored inverse diagonal)
-template <typename Real, int N, int NL, int T, int CP = 1>
+// two-CTA form: coefficients of coarse level NL from kappa in kin, coarser kappa into kout, then
+// recurse with the buffers swapped (no stored inverse diagonal)
+template <typename Real, int N, int NL, int T>
 __device__ void setup_levels_cp(Real* arena, Real* kin, Real* kout) {
-    Lv<Real> L = level_ptrs<Real, N, NL, CP>(arena);
+    Lv<Real> L = level_ptrs<Real, N, NL, true>(arena);
     build_coeffs<Real, NL, T>(L, kin);
     if constexpr (NL > 2) {
         coarsen_kappa<Real, NL / 2, T>(kin, kout);
         __syncthreads();
-        setup_levels_cp<Real, N, NL / 2, T, CP>(arena, kout, kin);
+        setup_levels_cp<Real, N, NL / 2, T>(arena, kout, kin);
     } else {
         __syncthreads();
     }
@@ -566,27 +526,22 @@ __host__ __device__ constexpr int solve_smem_reals(int N, int T) {
 
 // ---- the kernel ----------------------------------------------------------------------
 // the whole solve of particle p of a.n, by one thread block (all threads call it)
-// CP: compact hierarchy (mixed path, kappa from the synthesis) with the refinement state at
-// ref_ext (device memory) instead of shared memory. RHS: the load vector may come from a table
-// (a.rhs); false compiles the f = 1 path alone (the compact kernels are instantiated both ways:
-// at 64 registers a thread the table read's code costs them 20 % of their speed)
-template <typename Real, int N, int T, int CP = 0, bool RHS = true, bool FC = false>
+template <typename Real, int N, int T, bool FC = false>
 __device__ __forceinline__ void solve_particle(const FemArgs& a, const int p, Real* arena, double (*red_buf)[64],
-                                               Real* theta_s, Real* ref_ext = nullptr) {
+                                               Real* theta_s) {
     constexpr int S = Fine<Real, N>::S, NI = Fine<Real, N>::NI;
     constexpr int NPT = fine_slots(N, T, FC);          // slots per thread (colour_node positions)
     constexpr int NPH = NPT / 2;                       // per colour
     constexpr int E = 2 * N * N;
     const int tid = threadIdx.x;
 
-    Lv<Real> F = level_ptrs<Real, N, N, CP, FC>(arena);
+    Lv<Real> F = level_ptrs<Real, N, N, false, FC>(arena);
     Real* stage = F.e;     // e, res, p of the fine level are contiguous: 3*lvl_size(N) >= 2.5 N^2
-                           // (compact: e and p, 2*lvl_size(N) >= 2 N^2)
     if constexpr (FC) zero_ghost_weights<Real, N, N, T>(arena);   // read by the boundary rows
 
     // 1) kappa = exp(u) on every fine triangle: read from the tensor-core synthesis, or
     //    u = theta . Psi computed here (FP64 path)
-    if (CP || a.kappa) {
+    if (a.kappa) {
         const float* kp = a.kappa + (size_t)p * E;
         for (int e = tid; e < E; e += T) stage[e] = (Real)kp[e];
     } else {
@@ -602,33 +557,13 @@ __device__ __forceinline__ void solve_particle(const FemArgs& a, const int p, Re
     __syncthreads();
 
     // 2) stencil hierarchy
-    if constexpr (CP) {
-        // kappa ping-pongs between the fine level's e/p storage and its inverse-diagonal storage,
-        // which is filled last
-        build_coeffs<Real, N, T>(F, stage);
-        coarsen_kappa<Real, N / 2, T>(stage, F.iD);
-        __syncthreads();
-        setup_levels_cp<Real, N, N / 2, T>(arena, F.iD, stage);
-        build_diag<Real, N, T>(F);
-    } else {
-        setup_levels<Real, N, N, T, FC>(arena, stage, true);
-    }
-    zero_rings<Real, N, N, T, CP, FC>(arena);
+    setup_levels<Real, N, N, T, FC>(arena, stage, true);
+    zero_rings<Real, N, N, T, false, FC>(arena);
     __syncthreads();
-    Real* dinv = CP ? arena + arena_size_cp(N) : arena + arena_size(N, FC) + 4 * NPT * T;
-    if constexpr (direct_level<Real, FC>(N) != 0) {
-        if constexpr (CP) {
-            // compact forms: one warp runs the pivot steps while the SM's other blocks keep it busy
-            // (with one block per SM the block-wide form is faster)
-            if (tid < 32)
-                dense_setup<Real, direct_level<Real, FC>(N), 32, FC>(
-                    level_ptrs<Real, N, direct_level<Real, FC>(N), CP, FC>(arena), dinv);
-            __syncthreads();
-        } else {
-            dense_setup<Real, direct_level<Real, FC>(N), T, FC>(
-                level_ptrs<Real, N, direct_level<Real, FC>(N), CP, FC>(arena), dinv);
-        }
-    }
+    Real* dinv = arena + arena_size(N, FC) + 4 * NPT * T;
+    if constexpr (direct_level<Real, FC>(N) != 0)
+        dense_setup<Real, direct_level<Real, FC>(N), T, FC>(
+            level_ptrs<Real, N, direct_level<Real, FC>(N), false, FC>(arena), dinv);
 
     // fine nodes owned by this thread, one packed int each: bits 0-12 node index n, 13-23 the
     // coarse node c under it ((j/2) SC + i/2), 24-25 (i & 1) + 2 (j & 1), 26 red, 27 valid.
@@ -654,7 +589,7 @@ __device__ __forceinline__ void solve_particle(const FemArgs& a, const int p, Re
     // numbers on the mixed path so that no FP64 instruction runs in the solve. They are touched
     // once per refinement pass, so they live in shared memory after the arena ([4][NPT][T]:
     // x hi, x lo, r hi, r lo), conflict-free per slot.
-    Real* ref = CP ? ref_ext : arena + arena_size(N, FC);
+    Real* ref = arena + arena_size(N, FC);
     auto XH = [&](int q) -> Real& { return ref[(0 * NPT + q) * T + tid]; };
     auto XL = [&](int q) -> Real& { return ref[(1 * NPT + q) * T + tid]; };
     auto RH = [&](int q) -> Real& { return ref[(2 * NPT + q) * T + tid]; };
@@ -676,7 +611,7 @@ __device__ __forceinline__ void solve_particle(const FemArgs& a, const int p, Re
             bflow += RH(q) * RH(q);
         }
         block_sum<T>(bflow, red_buf[1]);
-    } else if (RHS && a.rhs) {
+    } else if (a.rhs) {
         // the load vector, read in a rolled loop of its own (node indices recomputed, no register
         // array touched), which leaves the register allocation of the solve as it is for f = 1
 #pragma unroll 1
@@ -694,7 +629,7 @@ __device__ __forceinline__ void solve_particle(const FemArgs& a, const int p, Re
     // inner CG state of this thread's nodes: residual r, correction d, preconditioned residual z
     // and search direction p (p is also published in shared memory for the stencil)
     Real r[NPT], d[NPT], z[NPT], pv[NPT];
-    const Real bnorm2 = FC ? bflow : (RHS && a.rhs) ? Real(a.bnorm2) : Real(NI) * h2 * h2;
+    const Real bnorm2 = FC ? bflow : a.rhs ? Real(a.bnorm2) : Real(NI) * h2 * h2;
     const Real stop_outer = Real(a.rtol * a.rtol) * bnorm2;
     // an inner pass ends at its relative reduction or once its residual is below half the outer
     // target, whichever comes first (the last pass then stops where the solve is done)
@@ -703,7 +638,7 @@ __device__ __forceinline__ void solve_particle(const FemArgs& a, const int p, Re
     int parity = 0;
     int total_it = 0;
     bool converged = false;
-    Lv<Real> C1 = level_ptrs<Real, N, N / 2, CP, FC>(arena);
+    Lv<Real> C1 = level_ptrs<Real, N, N / 2, false, FC>(arena);
     Real* P = F.rhs;   // fine-level CG direction (the fine rhs is r, held in registers)
 
     for (int pass = 0; pass < a.max_outer && !converged; ++pass) {
@@ -746,7 +681,7 @@ __device__ __forceinline__ void solve_particle(const FemArgs& a, const int p, Re
             __syncthreads();
             restrict_gather<Real, N / 2, T, FC>(F.res, C1);
             __syncthreads();
-            vcycle_coarse<Real, N, N / 2, T, false, CP, FC>(arena, dinv);
+            vcycle_coarse<Real, N, N / 2, T, false, false, FC>(arena, dinv);
 #pragma unroll
             for (int q = NPH; q < NPT; ++q) {
                 z[q] = Real(0);
@@ -1299,27 +1234,8 @@ fem_eval_kernel_fc(FemArgs a) {
     __shared__ double red_buf[2][64];
     __shared__ Real theta_s[256];
     if ((int)blockIdx.x >= a.n) return;
-    solve_particle<Real, N, T, false, false, true>(a, blockIdx.x, reinterpret_cast<Real*>(smem_raw), red_buf,
+    solve_particle<Real, N, T, true>(a, blockIdx.x, reinterpret_cast<Real*>(smem_raw), red_buf,
                                                    theta_s);
-}
-
-// compact form (mixed, kappa from the synthesis): MINB blocks per SM, persistent over the
-// particles; each block keeps its refinement state in its own slice of ref_scratch (L2-resident)
-template <int N, int T, int MINB, bool RHS>
-__global__ void __launch_bounds__(T, MINB) fem_eval_compact(FemArgs a, float* ref_scratch, int* counter) {
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    __shared__ double red_buf[2][64];
-    __shared__ int item_s;
-    float* ref = ref_scratch + (size_t)blockIdx.x * (4 * fine_slots(N, T) * T);
-    for (;;) {
-        if (threadIdx.x == 0) item_s = atomicAdd(counter, 1);
-        __syncthreads();
-        const int item = item_s;
-        __syncthreads();
-        if (item >= a.n) break;
-        solve_particle<float, N, T, true, RHS>(a, item, reinterpret_cast<float*>(smem_raw), red_buf, nullptr, ref);
-        __syncthreads();
-    }
 }
 
 // ---- two-CTA cluster form of the 1/128 solve (mixed path) ------------------------------------
@@ -1434,7 +1350,7 @@ __device__ void solve_particle_cl(const FemArgs& a, const int p, float* sm, floa
     const uint32_t pe = peer_addr(smem_addr(e), partner) + 4u * (uint32_t)shift;
     const uint32_t pres = peer_addr(smem_addr(res), partner) + 4u * (uint32_t)(shift / 2);
     const uint32_t pcb[2] = {peer_addr(smem_addr(cbuf[0]), partner), peer_addr(smem_addr(cbuf[1]), partner)};
-    const Lv<float> C1 = level_ptrs<float, N, N / 2, 2>(coarse);
+    const Lv<float> C1 = level_ptrs<float, N, N / 2, true>(coarse);
     const uint32_t pc_rhs = peer_addr(smem_addr(C1.rhs), partner), pc_e = peer_addr(smem_addr(C1.e), partner);
 
     // 1) stencil of the strip (local rows 0 .. 65 = rows 64 r .. 64 r + 65) straight from kappa,
@@ -1458,10 +1374,10 @@ __device__ void solve_particle_cl(const FemArgs& a, const int p, float* sm, floa
         aN[n] = 0.5f * an;
     }
     __syncthreads();
-    setup_levels_cp<float, N, N / 2, T, 2>(coarse, e, res);
+    setup_levels_cp<float, N, N / 2, T>(coarse, e, res);
     for (int n = tid; n < FS + RS; n += T) e[n] = 0.f;   // e and res (contiguous): zero halos and rings
-    zero_rings<float, N, N / 2, T, 2>(coarse);
-    if (tid < 32) dense_setup<float, 4, 32>(level_ptrs<float, N, 4, 2>(coarse), dinv);
+    zero_rings<float, N, N / 2, T, true>(coarse);
+    if (tid < 32) dense_setup<float, 4, 32>(level_ptrs<float, N, 4, true>(coarse), dinv);
     cluster_sync();   // also: the partner writes into this CTA's arrays only after they are zeroed
 
     unsigned slot[NPT];
@@ -1572,7 +1488,7 @@ __device__ void solve_particle_cl(const FemArgs& a, const int p, float* sm, floa
                 }
             }
             cluster_sync();
-            vcycle_coarse<float, N, N / 2, T, false, 2>(coarse, dinv);
+            vcycle_coarse<float, N, N / 2, T, false, true>(coarse, dinv);
             // black post-sweep with the prolongation folded in
 #pragma unroll
             for (int q = NPH; q < NPT; ++q) {
@@ -1875,47 +1791,6 @@ cudaError_t launch_global_multi(const FemArgs* groups, const int* offsets, const
     return cudaGetLastError();
 }
 
-// compiled compact configurations: blocks per SM that the registers are sized for (0: none)
-constexpr int compact_min_blocks(int N, int T) {
-    return (N == 64 && T == 512) ? 2 : (N == 32 && T == 256) ? 4 : 0;
-}
-
-template <int N>
-constexpr size_t compact_smem() {
-    return sizeof(float) * (size_t)(arena_size_cp(N) + dense_reals<float>(N));
-}
-
-template <int N, int T, bool RHS>
-cudaError_t launch_compact_t(const FemArgs& a, float* ref_scratch, int blocks, int* counter, cudaStream_t st) {
-    constexpr int MINB = compact_min_blocks(N, T);
-    cudaError_t e = cudaFuncSetAttribute(fem_eval_compact<N, T, MINB, RHS>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)compact_smem<N>());
-    if (e != cudaSuccess) return e;
-    fem_eval_compact<N, T, MINB, RHS><<<blocks, T, compact_smem<N>(), st>>>(a, ref_scratch, counter);
-    count_launches(1);
-    return cudaGetLastError();
-}
-
-template <int N, int T>
-cudaError_t launch_compact(const FemArgs& a, float* ref_scratch, int blocks, int* counter, cudaStream_t st) {
-    return a.rhs ? launch_compact_t<N, T, true>(a, ref_scratch, blocks, counter, st)
-                 : launch_compact_t<N, T, false>(a, ref_scratch, blocks, counter, st);
-}
-
-template <int N, int T>
-int compact_resident_blocks() {
-    constexpr int MINB = compact_min_blocks(N, T);
-    int dev = 0, sms = 0, per_sm = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    // the two instantiations share the launch bounds and the shared-memory size
-    cudaFuncSetAttribute(fem_eval_compact<N, T, MINB, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         (int)compact_smem<N>());
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fem_eval_compact<N, T, MINB, false>, T,
-                                                  compact_smem<N>());
-    return sms * std::max(1, per_sm);
-}
-
 // ---- two-CTA cluster form of 1/128 ----
 template <bool RHS>
 int cluster_resident_clusters() {
@@ -1945,20 +1820,6 @@ cudaError_t launch_cluster_t(const FemArgs& a, float* ref_scratch, int blocks, i
 
 }  // namespace
 
-int fem_compact_blocks(int N, int T) {
-    // resident blocks of a compact kernel, queried once per device and configuration
-    static int cached[64][2] = {};
-    const int c = (N == 64 && T == 512) ? 0 : (N == 32 && T == 256) ? 1 : -1;
-    if (c < 0) return 0;
-    int dev = 0;
-    cudaGetDevice(&dev);
-    if (dev >= 0 && dev < 64 && cached[dev][c] > 0) return cached[dev][c];
-    const int blocks = c == 0 ? compact_resident_blocks<64, 512>() : compact_resident_blocks<32, 256>();
-    if (dev >= 0 && dev < 64) cached[dev][c] = blocks;
-    return blocks;
-}
-size_t fem_compact_ref_floats(int N, int T) { return (size_t)4 * fine_slots(N, T) * T; }
-
 int fem_cluster_blocks() {
     // CTAs of the two-CTA form that are resident at once, queried once per device
     static int cached[64] = {};
@@ -1979,18 +1840,6 @@ cudaError_t fem_eval_cluster_launch(const FemArgs& a, float* ref_scratch, int bl
     if (e != cudaSuccess) return e;
     return a.rhs ? launch_cluster_t<true>(a, ref_scratch, grid, counter, st)
                  : launch_cluster_t<false>(a, ref_scratch, grid, counter, st);
-}
-
-cudaError_t fem_eval_compact_launch(const FemArgs& a, int T, float* ref_scratch, int blocks, int* counter,
-                                    cudaStream_t st) {
-    if (a.n <= 0) return cudaSuccess;
-    if (a.precision != SMC_MIXED || !a.kappa || compact_min_blocks(a.N, T) == 0) return cudaErrorInvalidValue;
-    const int grid = std::max(1, std::min(a.n, blocks));
-    cudaError_t e = cudaMemsetAsync(counter, 0, sizeof(int), st);
-    if (e != cudaSuccess) return e;
-    if (a.N == 64 && T == 512) return launch_compact<64, 512>(a, ref_scratch, grid, counter, st);
-    if (a.N == 32 && T == 256) return launch_compact<32, 256>(a, ref_scratch, grid, counter, st);
-    return cudaErrorInvalidValue;
 }
 
 size_t fem_global_slice(int N, bool FC) {
@@ -2039,6 +1888,11 @@ size_t fem_large_multi_scratch(int N) {
     return (size_t)fem_global_blocks(N) * fem_global_slice(N);
 }
 
+size_t fem_multi_scratch(int N, int precision) {
+    if (N >= 128) return fem_large_multi_scratch(N);
+    return fem_tile_form(N, precision, false) ? fem_tile_scratch(N) : 0;
+}
+
 cudaError_t fem_eval_large_multi_launch(int N, const FemArgs* groups, const int* offsets, const int* item_group,
                                         int total, float* scratch, int* counter, cudaStream_t st) {
     if (total <= 0) return cudaSuccess;
@@ -2075,10 +1929,6 @@ cudaError_t fem_eval_persistent_launch(int N, int precision, int T, const FemArg
             case 8 * 10000 + 32: return launch_persistent<float, 8, 32>(groups, offsets, item_group, total, counter, st);
             case 16 * 10000 + 128: return launch_persistent<float, 16, 128>(groups, offsets, item_group, total, counter, st);
             case 16 * 10000 + 64: return launch_persistent<float, 16, 64>(groups, offsets, item_group, total, counter, st);
-            case 32 * 10000 + 256: return launch_persistent<float, 32, 256>(groups, offsets, item_group, total, counter, st);
-            case 32 * 10000 + 512: return launch_persistent<float, 32, 512>(groups, offsets, item_group, total, counter, st);
-            case 64 * 10000 + 512: return launch_persistent<float, 64, 512>(groups, offsets, item_group, total, counter, st);
-            case 64 * 10000 + 1024: return launch_persistent<float, 64, 1024>(groups, offsets, item_group, total, counter, st);
         }
     } else {
         switch (N * 10000 + T) {
@@ -2098,9 +1948,8 @@ bool fem_level_supported(int N, int precision) {
     return N == 4 || N == 8 || N == 16 || N == 32;
 }
 
-// the block size used when none was chosen: the compact form where it is compiled (it is
-// faster at J = 4000 on 1/32 and 1/64, and bit-identical to the size -T), the two-CTA form on
-// 1/128, else the first size
+// the block size used when none was chosen: the two-CTA form on 1/128, else the first size; -512 and
+// -256 on 1/64 and 1/32, where every size names the register-tiled form (fem_tile.cu)
 int fem_default_block(int N, int precision) {
     if (precision == SMC_MIXED && (N == 32 || N == 64)) return N == 64 ? -512 : -256;
     // 1/128: the two-CTA cluster form where a cluster fits (1.2x the device-memory form at J = 4000
@@ -2117,8 +1966,8 @@ std::vector<int> fem_block_sizes(int N, int precision) {
             case 4: return {32};
             case 8: return {32, 64};
             case 16: return {128, 64};
-            case 32: return {256, 512, -256};   // -256: compact form, four blocks per SM
-            case 64: return {512, 1024, -512};  // -512: compact form, two blocks per SM
+            case 32: return {256, 512, -256};   // all: the register-tiled form
+            case 64: return {512, 1024, -512};
             case 128: return {1024, -1024};     // -1024: two-CTA cluster form (fine level on chip)
             case 256: return {1024};
         }
@@ -2160,10 +2009,6 @@ cudaError_t fem_eval_launch(const FemArgs& a, cudaStream_t st, int T) {
             case 8 * 10000 + 32: return launch_one<float, 8, 32>(a, st);
             case 16 * 10000 + 128: return launch_one<float, 16, 128>(a, st);
             case 16 * 10000 + 64: return launch_one<float, 16, 64>(a, st);
-            case 32 * 10000 + 256: return launch_one<float, 32, 256>(a, st);
-            case 32 * 10000 + 512: return launch_one<float, 32, 512>(a, st);
-            case 64 * 10000 + 512: return launch_one<float, 64, 512>(a, st);
-            case 64 * 10000 + 1024: return launch_one<float, 64, 1024>(a, st);
         }
     } else {
         switch (a.N * 10000 + T) {

@@ -62,14 +62,13 @@ struct FemArgs {
                             // (MIXED: hi, lo with hi + lo = the FP64 value); null: f = 1 (b = h^2)
     double bnorm2;          // sum of squares of the load vector over the interior nodes (with rhs)
     int flow_cell;          // 1: the flow cell of Example 5.3 (p = 0 / 1 on x = 0 / 1, no flow on
-                            // y = 0, 1, f = 0; levels 1/8 .. 1/256, FP64 to 1/32; no compact or
-                            // batched form)
+                            // y = 0, 1, f = 0; levels 1/8 .. 1/256, FP64 to 1/32; no batched form)
 };
 // Returns cudaSuccess or the launch error.
 // T = threads per particle (one of fem_block_sizes; <= 0: the first, the default)
 cudaError_t fem_eval_launch(const FemArgs& a, cudaStream_t stream, int T = 0);
 std::vector<int> fem_block_sizes(int N, int precision);
-// the size used when none is set (negative: a compact form)
+// the size used when none is set
 int fem_default_block(int N, int precision);
 // large levels (1/h = 128, 256; mixed precision, kappa from the synthesis): hierarchy in global
 // scratch, blocks x fem_global_slice(N) floats; *counter (device) is reset by the launch
@@ -86,14 +85,16 @@ cudaError_t fem_eval_global_multi_launch(int N, const FemArgs* groups, const int
 // items to the blocks
 cudaError_t fem_eval_persistent_launch(int N, int precision, int T, const FemArgs* groups, const int* offsets,
                                        const int* item_group, int total, int* counter, cudaStream_t st);
-// compact form of the mixed solve (negative block sizes of fem_block_sizes: -512 at 1/h = 64,
-// -256 at 1/h = 32): two or four blocks per SM, fem_compact_blocks(N, T) persistent blocks
-// (0 for a configuration that is not compiled) with fem_compact_ref_floats(N, T) floats of device
-// scratch each for the refinement state; *counter (device) is reset by the launch
-int fem_compact_blocks(int N, int T);
-size_t fem_compact_ref_floats(int N, int T);
-cudaError_t fem_eval_compact_launch(const FemArgs& a, int T, float* ref_scratch, int blocks, int* counter,
-                                    cudaStream_t st);
+// register-tiled form of the mixed Dirichlet solve on 1/64 and 1/32 (fem_tile.cu), every block size of
+// those levels: persistent blocks (2 of 256 threads an SM on 1/64, 8 of 64 on 1/32) with
+// fem_tile_scratch(N) floats of device scratch for their refinement state. *counter (device) is
+// reset by fem_tile_launch; fem_tile_multi_launch (arguments as fem_eval_persistent_launch) needs it
+// zero
+bool fem_tile_form(int N, int precision, bool flow_cell);
+size_t fem_tile_scratch(int N);
+cudaError_t fem_tile_launch(const FemArgs& a, float* scratch, int* counter, cudaStream_t st);
+cudaError_t fem_tile_multi_launch(int N, const FemArgs* groups, const int* offsets, const int* item_group, int total,
+                                  float* scratch, int* counter, cudaStream_t st);
 // two-CTA cluster form of the mixed 1/128 solve (block size -1024 of fem_block_sizes): the fine
 // level split in row strips over the two CTAs of a cluster, each on its own SM;
 // fem_cluster_blocks() CTAs (0 where no cluster fits) with fem_cluster_ref_floats() floats of
@@ -108,6 +109,8 @@ bool fem_cluster_form(int N, int precision, bool flow_cell);
 size_t fem_large_multi_scratch(int N);
 cudaError_t fem_eval_large_multi_launch(int N, const FemArgs* groups, const int* offsets, const int* item_group,
                                         int total, float* scratch, int* counter, cudaStream_t st);
+// device scratch (floats) of a many-problem launch on level N: the large levels', the tile form's, else 0
+size_t fem_multi_scratch(int N, int precision);
 bool fem_level_supported(int N, int precision);
 
 }  // namespace mls2mc
