@@ -20,7 +20,10 @@
 // fem_solve.cu) a node update reads nine words from shared memory, 21 block barriers an iteration; that
 // form (two 512-thread blocks an SM on 1/64) took 1.99 ms for 4000 particles on 1/64 and 0.42 ms on
 // 1/32. Here a patch of 16 nodes reads 8 rim words per half sweep, 16 barriers an iteration, 256 threads
-// of 128 registers, two blocks an SM (1/64) or 64 threads, eight blocks (1/32): 0.96 ms and 0.23 ms.
+// of 128 registers, two blocks an SM (1/64) or 64 threads, eight blocks (1/32): 0.76 ms and 0.16 ms.
+// What bounds it is latency: one 1/64 particle alone on an SM takes 0.87 of the time that two take
+// together. A spill is what hurts most: the direction p lives in shared memory and addresses are formed
+// where they are used, so that no register is spilled in the iteration (0.86 ms with a 20-word spill).
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -43,14 +46,16 @@ struct Geo {
     static constexpr int E = 0;              // sweep values, later p or d: rim positions [16][P]; the
                                              // inner positions' slots carry red residuals
     static constexpr int D = E + 16 * P;     // CG correction d, float4 [4][P] (set-up: coarse kappa)
-    static constexpr int ID = D + 16 * P;    // inverse diagonals, float4 [red 2, black 2][P]
+    static constexpr int PV = D + 16 * P;    // CG direction p, float4 [4][P] (not in registers during the V-cycle)
+    static constexpr int ID = PV + 16 * P;   // inverse diagonals, float4 [red 2, black 2][P]
     static constexpr int W1 = ID + 16 * P;   // next level: weights (E, W, N, S) of (0,0) (1,1) (1,0) (0,1)
     static constexpr int ID1 = W1 + 16 * P;  // its inverse diagonals, float2 [red, black][P]
     static constexpr int E1 = ID1 + 4 * P;   // its values, positions A + 2 B
     static constexpr int W2 = E1 + 4 * P;    // 1/16 (on 1/64): weights, inverse diagonal, values
     static constexpr int ID2 = W2 + (L2 ? 4 * P : 0);
     static constexpr int E2 = ID2 + (L2 ? P : 0);
-    static constexpr int W8 = E2 + (L2 ? P : 0);   // 1/8: weights float4 [64], inverse diagonal, values, rhs
+    static constexpr int R2 = E2 + (L2 ? P : 0);   // (1/16: red residuals)
+    static constexpr int W8 = R2 + (L2 ? P : 0);   // 1/8: weights float4 [64], inverse diagonal, values, rhs
     static constexpr int ID8 = W8 + 256, E8 = ID8 + 64, R8 = E8 + 64;
     static constexpr int E4 = R8 + 64;       // 1/4: values [4][4], rhs [9], dense inverse [9][9]
     static constexpr int R4 = E4 + 16, DINV = R4 + 16;
@@ -58,7 +63,6 @@ struct Geo {
     // set-up staging inside D: kappa of the next level [8][P], of the one below it [2][P], of 1/8
     // [2][64] (1/32: the previous one), of 1/4 [2][16]
     static constexpr int K1 = D, K2 = D + 8 * P, K8 = L2 ? D + 10 * P : K2, K4 = D + 10 * P + 128;
-    // Gauss-Jordan work of the 1/4 inverse (in E, before the first sweep)
     static constexpr int REF4 = 16 * P;      // float4s of refinement state of one block (device memory)
 };
 
@@ -91,66 +95,59 @@ __device__ __forceinline__ float off4(const float4 w, float e, float wv, float n
 }
 
 // inverse (row-major, symmetric) of the 9 x 9 operator of level 1/4 by Gauss-Jordan elimination
-// without pivoting (A is positive definite), one matrix entry per lane and step: lane l holds the
-// entries l, l + 32, l + 64 of the 81
-__device__ __forceinline__ void invert9(const float* k4, float* dinv, float* buf) {
-    const int lane = threadIdx.x & 31;
+// without pivoting (A is positive definite), by one warp: lane u < 9 keeps row u in registers, the pivot
+// row comes by shuffles. It is a serial chain that the block waits for: one matrix entry per lane in
+// shared memory with a branch per case took 12 K cycles, 9 % of the 1/64 solve.
+__device__ __forceinline__ void invert9(const float* k4, float* dinv) {
+    const int lane = threadIdx.x & 31, u = lane < 9 ? lane : 8;
     // kappa of the 4 x 4 cells: k4[2 c + t], c = J 4 + I, t = 0 lower, 1 upper half
     auto aE = [&](int I, int J) { return 0.5f * (k4[2 * (J * 4 + I)] + k4[2 * ((J - 1) * 4 + I) + 1]); };
     auto aN = [&](int I, int J) { return 0.5f * (k4[2 * (J * 4 + I - 1)] + k4[2 * (J * 4 + I) + 1]); };
-    float val[3];
+    const int I = u % 3 + 1, J = u / 3 + 1;
+    const float wE = aE(I, J), wW = aE(I - 1, J), wN = aN(I, J), wS = aN(I, J - 1);
+    float a[9];
 #pragma unroll
-    for (int q = 0; q < 3; ++q) {
-        const int idx = lane + 32 * q;
-        float x = 0.f;
-        if (idx < 81) {
-            const int u = idx / 9, v = idx - 9 * u;
-            const int ui = u % 3 + 1, uj = u / 3 + 1, vi = v % 3 + 1, vj = v / 3 + 1;
-            if (u == v) x = aE(ui, uj) + aE(ui - 1, uj) + aN(ui, uj) + aN(ui, uj - 1);
-            else if (uj == vj && vi == ui + 1) x = -aE(ui, uj);
-            else if (uj == vj && vi == ui - 1) x = -aE(ui - 1, uj);
-            else if (ui == vi && vj == uj + 1) x = -aN(ui, uj);
-            else if (ui == vi && vj == uj - 1) x = -aN(ui, uj - 1);
-            buf[idx] = x;
-        }
-        val[q] = x;
-    }
-    __syncwarp();
-    // step k reads row and column k of the current matrix from one buffer, writes the other
-#pragma unroll 1
+    for (int v = 0; v < 9; ++v)
+        a[v] = v == u ? wE + wW + wN + wS
+                      : v == u + 1 && I < 3 ? -wE : v == u - 1 && I > 1 ? -wW : v == u + 3 ? -wN : v == u - 3 ? -wS : 0.f;
+#pragma unroll
     for (int k = 0; k < 9; ++k) {
-        const float* cur = buf + (k & 1) * 96;
-        float* nxt = k == 8 ? dinv : buf + ((k + 1) & 1) * 96;
-        const float ip = 1.f / cur[10 * k];
+        float row[9];
 #pragma unroll
-        for (int q = 0; q < 3; ++q) {
-            const int idx = lane + 32 * q;
-            if (idx < 81) {
-                const int u = idx / 9, v = idx - 9 * u;
-                if (u == k) val[q] = v == k ? ip : cur[9 * k + v] * ip;
-                else if (v == k) val[q] = -cur[9 * u + k] * ip;
-                else val[q] = val[q] - cur[9 * u + k] * cur[9 * k + v] * ip;
-                nxt[idx] = val[q];
-            }
-        }
-        __syncwarp();
+        for (int v = 0; v < 9; ++v) row[v] = __shfl_sync(0xffffffffu, a[v], k);
+        const float ip = recip(row[k]);
+        const float f = u == k ? -ip : a[k] * ip;   // row k itself becomes row k / pivot
+#pragma unroll
+        for (int v = 0; v < 9; ++v) a[v] = v == k ? -f : fmaf(-f, row[v], u == k ? 0.f : a[v]);
     }
+    if (lane < 9)
+#pragma unroll
+        for (int v = 0; v < 9; ++v) dinv[9 * u + v] = a[v];
 }
 
 // the solve of particle `item` of a.n by the calling block (every thread of the block calls it).
-// sm: Geo<N>::FLOATS floats, red: [2][8] reduction buffers, ref: Geo<N>::REF4 float4 of device memory
+// sm: Geo<N>::FLOATS floats, red: [2][8] reduction buffers, part: [8], ref: Geo<N>::REF4 float4 of device memory
 // (this block's refinement state). RHS: the load vector may come from a table (a.rhs).
-template <int N, bool RHS>
-__device__ __forceinline__ void solve_tile(const FemArgs& a, const int item, float* sm, float (*red)[8], float4* ref) {
+// take(): called by the block's last thread while the observations are formed (the next ticket).
+template <int N, bool RHS, typename Take>
+__device__ __forceinline__ void solve_tile(const FemArgs& a, const int item, float* sm, float (*red)[8], double* part,
+                                           float4* ref, Take&& take) {
     using G = Geo<N>;
     constexpr int P = G::P, TX = G::TX, NW = G::NW;
     const int tid = threadIdx.x, lane = tid & 31;
     const int tx = tid % TX, ty = tid / TX;
     // neighbouring patches (wrapped; see above)
     const int pL = (tid - 1) & (P - 1), pR = (tid + 1) & (P - 1), pB = (tid - TX) & (P - 1), pA = (tid + TX) & (P - 1);
-    const int pD = (tid - TX - 1) & (P - 1), pU = (tid + TX + 1) & (P - 1);
+    // the diagonal ones, formed where they are used (opaque to the compiler, which would otherwise keep
+    // them and the addresses derived from them in registers through the iteration and spill)
+    auto diagonal = [&](int off) {
+        int t = tid;
+        asm volatile("" : "+r"(t));
+        return (t + off) & (P - 1);
+    };
     float* E = sm + G::E;
     float4* D4 = reinterpret_cast<float4*>(sm + G::D);
+    float4* PV4 = reinterpret_cast<float4*>(sm + G::PV);
     float4* ID4 = reinterpret_cast<float4*>(sm + G::ID);
     float4* W1 = reinterpret_cast<float4*>(sm + G::W1);
     float2* ID1 = reinterpret_cast<float2*>(sm + G::ID1);
@@ -223,6 +220,7 @@ __device__ __forceinline__ void solve_tile(const FemArgs& a, const int item, flo
     __syncthreads();
     {   // next level: the weights of the 2 x 2 nodes
         float lo[3][3], up[3][3];   // cells (-1 .. 1)^2, index [row + 1][column + 1]
+        const int pD = diagonal(-TX - 1);
         auto K = [&](int pos, int t, int p) { return sm[G::K1 + (2 * pos + t) * P + p]; };
         lo[1][0] = K(1, 0, pL); up[1][0] = K(1, 1, pL); lo[2][0] = K(3, 0, pL);
         lo[0][0] = K(3, 0, pD); up[0][0] = K(3, 1, pD);
@@ -286,7 +284,7 @@ __device__ __forceinline__ void solve_tile(const FemArgs& a, const int item, flo
             E4[lane] = 0.f;
         }
         __syncwarp();
-        invert9(k4, DI, sm + G::K4 + 32);
+        invert9(k4, DI);
     }
 
     // ---- rim exchange: colour c's values of the neighbouring patches next to the patch's other colour
@@ -303,7 +301,7 @@ __device__ __forceinline__ void solve_tile(const FemArgs& a, const int item, flo
             }
         }
     };
-    float r[4][4], p[4][4], e[4][4];
+    float r[4][4], e[4][4];
     auto store_rim = [&](int c, const float (&v)[4][4]) {   // c = 2: both colours
 #pragma unroll
         for (int b = 0; b < 4; ++b)
@@ -341,6 +339,7 @@ __device__ __forceinline__ void solve_tile(const FemArgs& a, const int item, flo
     int parity = 0, total_it = 0;
     bool converged = false, have_x = false;
 
+#pragma unroll 1
     for (int pass = 0; pass < a.max_outer && !converged; ++pass) {
         float rr = 0.f;
 #pragma unroll
@@ -373,6 +372,7 @@ __device__ __forceinline__ void solve_tile(const FemArgs& a, const int item, flo
         if (!(rr0 > 0.f)) break;
         const float stop2 = fmaxf(rtol_in2 * rr0, stop_last);
         float rz = 0.f;
+#pragma unroll 1
         for (int it = 0; it < a.max_inner; ++it) {
             // black pre-sweep
             load_halo(0);
@@ -398,7 +398,7 @@ __device__ __forceinline__ void solve_tile(const FemArgs& a, const int item, flo
                 E[6 * P + tid] = s13;
                 E[9 * P + tid] = s31;
                 __syncthreads();
-                v00 = s00 + 0.5f * (s11 + E[5 * P + pD]);
+                v00 = s00 + 0.5f * (s11 + E[5 * P + diagonal(-TX - 1)]);
                 v10 = s20 + 0.5f * (s31 + E[6 * P + pB]);
                 v01 = s02 + 0.5f * (s13 + E[9 * P + pL]);
                 v11 = s22 + 0.5f * (s33 + s11);
@@ -422,6 +422,7 @@ __device__ __forceinline__ void solve_tile(const FemArgs& a, const int item, flo
             __syncthreads();
             float v2;   // right-hand side of the node (tx, ty) two levels down
             {
+                const int pD = diagonal(-TX - 1);
                 const float l10 = E1[P + pL], b01 = E1[2 * P + pB];
                 const float s00 = off4(W1[tid], e10, l10, e01, b01);
                 const float s11 = off4(W1[P + tid], E1[2 * P + pR], e01, E1[P + pA], e10);
@@ -441,24 +442,28 @@ __device__ __forceinline__ void solve_tile(const FemArgs& a, const int item, flo
                     E2[tid] = e2;
                 }
                 __syncthreads();
+                // every node's residual once (red: the off-diagonal sum; a black node's is not used), so
+                // that warp 0 only adds up three values per node of 1/8
+                sm[G::R2 + tid] = off4(W2[tid], E2[pR], E2[pL], E2[pA], E2[pB]);
+                __syncthreads();
             } else {
                 R8[tid] = v2;
                 if (red2) E8[tid] = v2 * ID8[tid];
                 __syncthreads();
             }
             if (tid < 32) {   // levels 1/8 and 1/4 in warp 0; node c = 8 J + I
-                const int J = lane >> 2;
-                const int cr = 8 * J + 2 * (lane & 3) + (J & 1), cb = cr ^ 1;   // this lane's red and black node
+                // the lane made opaque: the addresses below are computed here instead of being hoisted
+                // out of the iteration into registers that do not exist (spills)
+                int ln = lane;
+                asm volatile("" : "+r"(ln));
+                const int J = ln >> 2;
+                const int cr = 8 * J + 2 * (ln & 3) + (J & 1), cb = cr ^ 1;   // this ln's red and black node
                 float rr8, rb8;
                 if constexpr (G::L2) {
-                    auto s16 = [&](int f) {   // red residual at node f of 1/16
-                        f &= P - 1;
-                        return off4(W2[f], E2[(f + 1) & (P - 1)], E2[(f - 1) & (P - 1)], E2[(f + TX) & (P - 1)],
-                                    E2[(f - TX) & (P - 1)]);
-                    };
+                    const float* R2 = sm + G::R2;
                     const int fr = 2 * J * TX + 2 * (cr & 7), fb = 2 * J * TX + 2 * (cb & 7);
-                    rr8 = s16(fr) + 0.5f * (s16(fr + TX + 1) + s16(fr - TX - 1));
-                    rb8 = s16(fb) + 0.5f * (s16(fb + TX + 1) + s16(fb - TX - 1));
+                    rr8 = R2[fr] + 0.5f * (R2[fr + TX + 1] + R2[(fr - TX - 1) & (P - 1)]);
+                    rb8 = R2[fb] + 0.5f * (R2[fb + TX + 1] + R2[(fb - TX - 1) & (P - 1)]);
                     E8[cr] = rr8 * ID8[cr];
                     __syncwarp();
                 } else {
@@ -470,16 +475,18 @@ __device__ __forceinline__ void solve_tile(const FemArgs& a, const int item, flo
                 };
                 E8[cb] = (rb8 + s8(cb)) * ID8[cb];
                 __syncwarp();
-                if (lane < 9) {
-                    const int f = (lane / 3 + 1) * 16 + (lane % 3 + 1) * 2;
-                    R4[lane] = s8(f) + 0.5f * (s8(f + 9) + s8(f - 9));
+                R8[cr] = s8(cr);   // red residuals
+                __syncwarp();
+                if (ln < 9) {
+                    const int f = (ln / 3 + 1) * 16 + (ln % 3 + 1) * 2;
+                    R4[ln] = R8[f] + 0.5f * (R8[f + 9] + R8[f - 9]);
                 }
                 __syncwarp();
-                if (lane < 9) {   // 1/4 solved exactly (the inverse is symmetric: column reads)
+                if (ln < 9) {   // 1/4 solved exactly (the inverse is symmetric: column reads)
                     float acc = 0.f;
 #pragma unroll
-                    for (int v = 0; v < 9; ++v) acc = fmaf(DI[9 * v + lane], R4[v], acc);
-                    E4[(lane / 3 + 1) * 4 + lane % 3 + 1] = acc;
+                    for (int v = 0; v < 9; ++v) acc = fmaf(DI[9 * v + ln], R4[v], acc);
+                    E4[(ln / 3 + 1) * 4 + ln % 3 + 1] = acc;
                 }
                 __syncwarp();
                 {   // black post-sweep with the prolongation
@@ -517,7 +524,7 @@ __device__ __forceinline__ void solve_tile(const FemArgs& a, const int item, flo
                 e2s = E8;
             }
             {   // 2 x 2 level, black post-sweep: red neighbours with the correction of the level below
-                const float c0 = e2s[tid], cR = e2s[pR], cA = e2s[pA], cU = e2s[pU], cL = e2s[pL], cB = e2s[pB];
+                const float c0 = e2s[tid], cR = e2s[pR], cA = e2s[pA], cU = e2s[diagonal(TX + 1)], cL = e2s[pL], cB = e2s[pB];
                 const float2 idb = ID1[P + tid];
                 const float f00 = e00 + c0, f11 = e11 + 0.5f * (c0 + cU);
                 const float fR = E1[pR] + cR, fA = E1[pA] + cA;
@@ -538,7 +545,7 @@ __device__ __forceinline__ void solve_tile(const FemArgs& a, const int item, flo
             __syncthreads();
             {   // fine black post-sweep: red values plus the prolonged correction
                 load_halo(0);
-                const float c20 = E1[pR], c21 = E1[2 * P + pR], c02 = E1[pA], c12 = E1[P + pA], c22 = E1[pU];
+                const float c20 = E1[pR], c21 = E1[2 * P + pR], c02 = E1[pA], c12 = E1[P + pA], c22 = E1[diagonal(TX + 1)];
                 const float cm0 = E1[P + pL], cm1 = E1[3 * P + pL], c0m = E1[2 * P + pB], c1m = E1[3 * P + pB];
                 e[0][0] += e00;
                 e[0][2] += e10;
@@ -585,10 +592,20 @@ __device__ __forceinline__ void solve_tile(const FemArgs& a, const int item, flo
             parity ^= 1;
             const float beta = it == 0 ? 0.f : rz_new / rz;
             rz = rz_new;
+            float p[4][4];   // p = z + beta p
 #pragma unroll
-            for (int b = 0; b < 4; ++b)
-#pragma unroll
-                for (int i = 0; i < 4; ++i) p[b][i] = it == 0 ? e[b][i] : e[b][i] + beta * p[b][i];
+            for (int b = 0; b < 4; ++b) {
+                float4 v = make_float4(e[b][0], e[b][1], e[b][2], e[b][3]);
+                if (it > 0) {
+                    const float4 o = PV4[b * P + tid];
+                    v.x += beta * o.x;
+                    v.y += beta * o.y;
+                    v.z += beta * o.z;
+                    v.w += beta * o.w;
+                }
+                PV4[b * P + tid] = v;
+                p[b][0] = v.x; p[b][1] = v.y; p[b][2] = v.z; p[b][3] = v.w;
+            }
             store_rim(2, p);
             __syncthreads();
             // q = A p in edge form (into e), alpha = rz / p.q
@@ -641,6 +658,7 @@ __device__ __forceinline__ void solve_tile(const FemArgs& a, const int item, flo
             if (!(rr > stop2)) break;   // also leaves on NaN
         }
         // ---- refinement: x += d, r -= A d in double-float arithmetic (edge form) ----
+        float p[4][4];   // d
 #pragma unroll
         for (int b = 0; b < 4; ++b) {
             const float4 d = D4[b * P + tid];
@@ -651,6 +669,18 @@ __device__ __forceinline__ void solve_tile(const FemArgs& a, const int item, flo
         load_halo(0);
         load_halo(1);
         float rr_out = 0.f;
+        // flux w (d_i - d_j) of an edge as an exact-difference, exact-product pair; an edge inside the patch
+        // is computed once and enters its two nodes with opposite signs (negation is exact)
+        auto flux = [](float w, float di, float dj, float& ph, float& pl) {
+            float sh, sl;
+            two_sum(di, -dj, sh, sl);    // d_i - d_j exactly
+            ph = __fmul_rn(w, sh);       // kept out of FMA contraction
+            pl = fmaf(w, sh, -ph);       // exact product error
+            pl = fmaf(w, sl, pl);
+        };
+        float sth[4], stl[4];   // fluxes through the patch rows' lower edges (node below -> node)
+#pragma unroll
+        for (int i = 0; i < 4; ++i) flux(wN[0][i], hB[i], p[0][i], sth[i], stl[i]);
 #pragma unroll
         for (int b = 0; b < 4; ++b) {
             float rh[4], rl[4], xh[4], xl[4];
@@ -658,7 +688,8 @@ __device__ __forceinline__ void solve_tile(const FemArgs& a, const int item, flo
 #pragma unroll
                 for (int i = 0; i < 4; ++i) {
                     load_b(i, b, rh[i], rl[i]);
-                    xh[i] = xl[i] = 0.f;
+                    xh[i] = p[b][i];
+                    xl[i] = 0.f;
                 }
             } else {
                 const float4 v0 = ref[b * P + tid], v1 = ref[(4 + b) * P + tid], v2 = ref[(8 + b) * P + tid],
@@ -667,27 +698,34 @@ __device__ __forceinline__ void solve_tile(const FemArgs& a, const int item, flo
                 rl[0] = v1.x; rl[1] = v1.y; rl[2] = v1.z; rl[3] = v1.w;
                 xh[0] = v2.x; xh[1] = v2.y; xh[2] = v2.z; xh[3] = v2.w;
                 xl[0] = v3.x; xl[1] = v3.y; xl[2] = v3.z; xl[3] = v3.w;
+#pragma unroll
+                for (int i = 0; i < 4; ++i) df_add(xh[i], xl[i], p[b][i], 0.f);
             }
+            float wsh, wsl;   // flux through the left edge of the node (left node -> node)
+            flux(wE[b][0], hL[b], p[b][0], wsh, wsl);
 #pragma unroll
             for (int i = 0; i < 4; ++i) {
-                const float di = p[b][i];
-                const float w[4] = {wE[b][i + 1], wE[b][i], wN[b + 1][i], wN[b][i]};
-                const float dj[4] = {i < 3 ? p[b][i < 3 ? i + 1 : 3] : hR[b], i > 0 ? p[b][i > 0 ? i - 1 : 0] : hL[b],
-                                     b < 3 ? p[b < 3 ? b + 1 : 3][i] : hA[i], b > 0 ? p[b > 0 ? b - 1 : 0][i] : hB[i]};
-                float ah = 0.f, al = 0.f;
-#pragma unroll
-                for (int t = 0; t < 4; ++t) {
-                    float sh, sl;
-                    two_sum(di, -dj[t], sh, sl);           // d_i - d_j exactly
-                    const float ph = __fmul_rn(w[t], sh);  // kept out of FMA contraction
-                    float pl = fmaf(w[t], sh, -ph);        // exact product error
-                    pl = fmaf(w[t], sl, pl);
-                    df_add(ah, al, ph, pl);
-                }
-                if (dirichlet(i, b)) ah = al = 0.f;
-                df_add(rh[i], rl[i], -ah, -al);
-                df_add(xh[i], xl[i], di, 0.f);
+                float eh, el, nh, nl;
+                flux(wE[b][i + 1], p[b][i], i < 3 ? p[b][i < 3 ? i + 1 : 3] : hR[b], eh, el);
+                flux(wN[b + 1][i], p[b][i], b < 3 ? p[b < 3 ? b + 1 : 3][i] : hA[i], nh, nl);
+                // r -= (east + north) - (west + south): high parts by TwoSum, the rest in one low part
+                float h = rh[i], l = rl[i], t;
+                two_sum(h, -eh, h, t);
+                l += t - el;
+                two_sum(h, wsh, h, t);
+                l += t + wsl;
+                two_sum(h, -nh, h, t);
+                l += t - nl;
+                two_sum(h, sth[i], h, t);
+                l += t + stl[i];
+                rh[i] = h + l;
+                rl[i] = l - (rh[i] - h);
+                if (dirichlet(i, b)) rh[i] = rl[i] = 0.f;
                 rr_out += rh[i] * rh[i];
+                wsh = eh;
+                wsl = el;
+                sth[i] = nh;
+                stl[i] = nl;
             }
             ref[b * P + tid] = make_float4(rh[0], rh[1], rh[2], rh[3]);
             ref[(4 + b) * P + tid] = make_float4(rl[0], rl[1], rl[2], rl[3]);
@@ -716,79 +754,78 @@ __device__ __forceinline__ void solve_tile(const FemArgs& a, const int item, flo
         xs[(4 * b + 3) * P + tid] = make_float2(xh.w, xl.w);
     }
     __syncthreads();
-    if (tid < 32) {
-        auto val = [&](int n) -> double {   // n = j (N + 2) + i
-            const int j = n / fem_row_stride(N), i = n - j * fem_row_stride(N);
-            if (i < 1 || i >= N || j < 1 || j >= N) return 0.0;
-            const float2 v = xs[(4 * (j & 3) + (i & 3)) * P + (j >> 2) * TX + (i >> 2)];
-            return (double)v.x + (double)v.y;
-        };
-        double misfit = 0.0;
-        for (int o = lane; o < a.n_obs; o += 32) {
-            const double g = a.obs_w[3 * o] * val(a.obs_idx[3 * o]) + a.obs_w[3 * o + 1] * val(a.obs_idx[3 * o + 1]) +
-                             a.obs_w[3 * o + 2] * val(a.obs_idx[3 * o + 2]);
-            if (a.G) a.G[(size_t)item * a.n_obs + o] = g;
-            const double rdf = a.y[o] - g;
-            misfit += rdf * rdf;
-        }
+    auto val = [&](int n) -> double {   // n = j (N + 2) + i
+        const int j = n / fem_row_stride(N), i = n - j * fem_row_stride(N);
+        if (i < 1 || i >= N || j < 1 || j >= N) return 0.0;
+        const float2 v = xs[(4 * (j & 3) + (i & 3)) * P + (j >> 2) * TX + (i >> 2)];
+        return (double)v.x + (double)v.y;
+    };
+    if (tid == G::T - 1) take();   // the ticket's latency overlaps the observations
+    double misfit = 0.0;
+    for (int o = tid; o < a.n_obs; o += G::T) {
+        const double g = a.obs_w[3 * o] * val(a.obs_idx[3 * o]) + a.obs_w[3 * o + 1] * val(a.obs_idx[3 * o + 1]) +
+                         a.obs_w[3 * o + 2] * val(a.obs_idx[3 * o + 2]);
+        if (a.G) a.G[(size_t)item * a.n_obs + o] = g;
+        const double rdf = a.y[o] - g;
+        misfit += rdf * rdf;
+    }
+    const int nw = min(NW, (a.n_obs + 31) / 32);   // warps that hold observations
+    if (tid < 32 * nw) {
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) misfit += __shfl_xor_sync(0xffffffffu, misfit, o);
-        if (tid == 0) {
-            a.Phi[item] = 0.5 * misfit * a.inv_sigma2;
-            if (a.iters) a.iters[item] = converged ? total_it : -(total_it + 1);
-        }
+        if (lane == 0) part[tid >> 5] = misfit;
+    }
+    __syncthreads();
+    if (tid == 0) {
+        for (int k = 1; k < nw; ++k) misfit += part[k];
+        a.Phi[item] = 0.5 * misfit * a.inv_sigma2;
+        if (a.iters) a.iters[item] = converged ? total_it : -(total_it + 1);
     }
 }
 
-// persistent blocks take particles from a ticket counter; thread 0 takes the next ticket before the
-// solve of the current one, so the atomic's latency is hidden
+// persistent blocks take particles from a ticket counter
 template <int N, bool RHS>
 __global__ void __launch_bounds__(Geo<N>::T, Geo<N>::MINB) fem_tile_kernel(FemArgs a, float4* ref_scratch, int* counter) {
     extern __shared__ __align__(16) float sm[];
     __shared__ __align__(16) float red[2][8];
+    __shared__ double part[8];
     __shared__ int item_s;
     float4* ref = ref_scratch + (size_t)blockIdx.x * Geo<N>::REF4;
-    int next = 0;
-    if (threadIdx.x == 0) next = atomicAdd(counter, 1);
+    if (threadIdx.x == 32) item_s = atomicAdd(counter, 1);
+    __syncthreads();
     for (;;) {
-        if (threadIdx.x == 0) {
-            item_s = next;
-            if (next < a.n) next = atomicAdd(counter, 1);
-        }
-        __syncthreads();
         const int item = item_s;
         if (item >= a.n) break;
-        solve_tile<N, RHS>(a, item, sm, red, ref);
+        solve_tile<N, RHS>(a, item, sm, red, part, ref, [&] { item_s = atomicAdd(counter, 1); });
         __syncthreads();
     }
 }
 
 // many problems: the same loop over (problem, particle) items; the item's launch arguments are copied
-// to shared memory
+// to shared memory (two copies: the next item's arrive while the current one's are in use)
 template <int N>
 __global__ void __launch_bounds__(Geo<N>::T, Geo<N>::MINB)
     fem_tile_multi(const FemArgs* groups, const int* offsets, const int* item_group, int total, float4* ref_scratch,
                    int* counter) {
     extern __shared__ __align__(16) float sm[];
     __shared__ __align__(16) float red[2][8];
-    __shared__ int item_s, p_s;
-    __shared__ FemArgs args_s;
+    __shared__ double part[8];
+    __shared__ int item_s[2], p_s[2];
+    __shared__ FemArgs args_s[2];
     float4* ref = ref_scratch + (size_t)blockIdx.x * Geo<N>::REF4;
-    int next = 0;
-    if (threadIdx.x == 0) next = atomicAdd(counter, 1);
-    for (;;) {
-        if (threadIdx.x == 0) {
-            item_s = next;
-            if (next < total) {
-                const int g = item_group[next];
-                args_s = groups[g];
-                p_s = next - offsets[g];
-                next = atomicAdd(counter, 1);
-            }
+    auto take = [&](int k) {
+        const int item = atomicAdd(counter, 1);
+        item_s[k] = item;
+        if (item < total) {
+            const int g = item_group[item];
+            args_s[k] = groups[g];
+            p_s[k] = item - offsets[g];
         }
-        __syncthreads();
-        if (item_s >= total) break;
-        solve_tile<N, true>(args_s, p_s, sm, red, ref);
+    };
+    if (threadIdx.x == 32) take(0);
+    __syncthreads();
+    for (int k = 0; item_s[k] < total; k ^= 1) {
+        solve_tile<N, true>(args_s[k], p_s[k], sm, red, part, ref, [&] { take(k ^ 1); });
         __syncthreads();
     }
 }
