@@ -81,8 +81,8 @@ extern "C" {
 typedef struct {
     int n_levels;              /* N_L >= 1 */
     const int* inv_h;          /* [n_levels] 1/h_l, coarse to fine; powers of two in [4, 32] (FP64),
-                                  [4, 256] (mixed; 1/128 keeps its fine level on chip across the two
-                                  CTAs of a thread-block cluster, 1/256 in device memory) */
+                                  [4, 256] (mixed; 1/128 and 1/256 keep their fine levels on chip across
+                                  the two or eight CTAs of a thread-block cluster) */
     int K;                     /* KL terms N_sto: 1 <= K <= 256, or <= 512 with the FEM forward map at
                                   SMC_MIXED (Example 5.3 keeps 320); Matern: K <= 512 */
     double corr_len;           /* correlation length of the separable exponential covariance */
@@ -187,11 +187,13 @@ int smc_set_timing(smc_handle* h, int enable);
  * block size for a level (T = 0 restores the default: -512 and -256 on 1/64 and 1/32 of the mixed
  * path, the two-CTA form on 1/128, else the first compiled size); T must be one of the
  * compiled sizes. On 1/64 (512, 1024, -512) and 1/32 (256, 512, -256) of the mixed path every size
+ * compiled sizes. On 1/64 (512, 1024, -512) and 1/32 (256, 512, -256) of the mixed path every size
  * names the same register-tiled form (two particles per SM on 1/64, eight on 1/32; the flow cell has one
  * form per level of its own). At 1/h = 128, -1024 selects the two-CTA form: one particle per cluster of
- * two CTAs of 1024 threads on two SMs, each keeping half of the fine rows on chip with one halo row
- * from the other through distributed shared memory, the coarse levels 1/64 .. 1/2 in both (the same
- * algorithm as 1024, which keeps the fine level in device memory; potentials agree to rounding).
+ * two CTAs of 512 threads on two SMs, each with half of the two finest levels on chip, border rows
+ * exchanged through distributed shared memory, the levels 1/32 .. 1/2 in both (the same
+ * algorithm as 1024, which keeps the fine level in device memory; potentials agree to rounding). 1/256 runs
+ * on clusters of eight such CTAs, or in the device-memory form where none fits.
  * Batched solves on 1/128 run the two-CTA form where a cluster fits; flow-cell solves the
  * device-memory form. */
 int smc_autotune(smc_handle* h, int n_tune, int* chosen, float* best_ms);
@@ -221,9 +223,8 @@ int smc_sizes(const smc_handle* h, int* K, int* n_obs, int* n_levels, int* J);
  * theta[p], [n[p]][K_p]) on its level level[p], writing phi[p] [n[p]] (device) and, if iters is
  * not NULL, iters[p] [n[p]] (device, as in smc_eval_likelihood_device): the tensor-core KL
  * syntheses of all mixed-precision problems, then one persistent solve launch per level size
- * whose blocks take (problem, particle) work items from a device counter (1/h = 128 in the two-CTA
- * form, whose clusters take the items, where a cluster fits; 1/h = 256 in the form that keeps its
- * fine levels in device memory). With use_graph = 1 the
+ * whose blocks (1/h = 128 and 256: clusters) take (problem, particle) work items from a device
+ * counter. With use_graph = 1 the
  * sequence is captured into a CUDA graph on `stream` (which must not be the default stream) the
  * first time and replayed afterwards, as long as levels, counts and pointers are unchanged. The
  * call queues work on `stream` and does not wait. Handles must be distinct FEM handles and must

@@ -35,12 +35,12 @@ int enqueue(Batch* b, const int* level, const int* n, const double* const* theta
     cudaError_t e = cudaMemsetAsync(b->d_counters, 0, sizeof(int) * b->groups.size(), st);
     for (size_t g = 0; g < b->groups.size() && e == cudaSuccess; ++g) {
         const auto& G = b->groups[g];
-        if (G.N >= 128)   // the form single solves default to (two-CTA on 1/128)
-            e = fem_eval_large_multi_launch(G.N, G.d_args, G.d_offsets, G.d_item_group, G.total, b->big_scratch,
-                                            b->d_counters + g, st);
-        else if (fem_tile_form(G.N, G.precision, false))
+        if (fem_tile_form(G.N, G.precision, false))   // the form single solves default to
             e = fem_tile_multi_launch(G.N, G.d_args, G.d_offsets, G.d_item_group, G.total, b->big_scratch,
                                       b->d_counters + g, st);
+        else if (G.N >= 128)
+            e = fem_eval_global_multi_launch(G.N, G.d_args, G.d_offsets, G.d_item_group, G.total, b->big_scratch,
+                                             fem_global_blocks(G.N), b->d_counters + g, st);
         else
             e = fem_eval_persistent_launch(G.N, G.precision, G.T, G.d_args, G.d_offsets, G.d_item_group, G.total,
                                            b->d_counters + g, st);

@@ -196,13 +196,13 @@ int multi_eval(Batch* b, const std::vector<EvalReq>& reqs, cudaStream_t st) {
         cudaError_t e = cudaGetLastError();
         for (size_t gi = 0; gi < groups.size() && e == cudaSuccess; ++gi) {
             const G& g = groups[gi];
-            if (g.N >= 128)   // the form single solves default to (two-CTA on 1/128)
-                e = fem_eval_large_multi_launch(g.N, S->d_args + g.first, S->d_offsets + g.first,
-                                                S->d_item_group + g.item_base, g.total, S->big_scratch,
-                                                S->d_counters + gi, st);
-            else if (fem_tile_form(g.N, g.precision, false))
+            if (fem_tile_form(g.N, g.precision, false))   // the form single solves default to
                 e = fem_tile_multi_launch(g.N, S->d_args + g.first, S->d_offsets + g.first,
                                           S->d_item_group + g.item_base, g.total, S->big_scratch, S->d_counters + gi, st);
+            else if (g.N >= 128)
+                e = fem_eval_global_multi_launch(g.N, S->d_args + g.first, S->d_offsets + g.first,
+                                                 S->d_item_group + g.item_base, g.total, S->big_scratch,
+                                                 fem_global_blocks(g.N), S->d_counters + gi, st);
             else
                 e = fem_eval_persistent_launch(g.N, g.precision, g.T, S->d_args + g.first, S->d_offsets + g.first,
                                                S->d_item_group + g.item_base, g.total, S->d_counters + gi, st);

@@ -31,10 +31,9 @@
 // vectors e (multigrid correction), res (residual) and rhs (fine level: the CG
 // direction p). The fine-level CG vectors r, d, z, p of a thread's nodes live in
 // registers (every fine node belongs to one thread for the whole solve); the
-// refinement state x, r (double-float pairs) lives in shared memory. The mixed Dirichlet solve on 1/64
-// and 1/32 has a form of its own (fem_tile.cu). Level 1/128 is solved by a cluster of two CTAs
-// on two SMs, each keeping half of the fine rows on chip (fem_eval_cluster); levels 1/128 (block
-// size 1024, the flow cell) and 1/256 can keep their two finest levels in device memory
+// refinement state x, r (double-float pairs) lives in shared memory. The mixed Dirichlet solve on 1/32 ..
+// 1/256 has a form of its own (fem_tile.cu); the flow cell's on 1/128 and 1/256, and the Dirichlet problem's at
+// block size 1024 on 1/128 or where no cluster fits, keep the two finest levels in device memory
 // (fem_eval_global).
 #include <cuda_runtime.h>
 
@@ -69,15 +68,7 @@ struct Lv {
     Real *aE, *aN, *iD, *e, *res, *rhs;   // iD: inverse of the stencil diagonal
 };
 
-// Coarse hierarchy of the two-CTA form (levels N/2 .. 2): four arrays a level (aE, aN, e, rhs: no res,
-// and the inverse diagonal is formed from the edge weights where a sweep needs it).
-__host__ __device__ constexpr int coarse_size_cp(int NL) { return NL < 2 ? 0 : 4 * lvl_size(NL) + coarse_size_cp(NL / 2); }
-__host__ __device__ constexpr int coarse_offset_cp(int NL, int NC) {
-    return NL == NC ? 0 : 4 * lvl_size(NL) + coarse_offset_cp(NL / 2, NC);
-}
-
-// CP: the coarse hierarchy of the two-CTA form (NL < N), from the arena's start
-template <typename Real, int N, int NL, bool CP = false, bool FC = false>
+template <typename Real, int N, int NL, bool FC = false>
 __device__ __forceinline__ Lv<Real> level_ptrs(Real* arena) {
     if constexpr (FC) {   // ghost row -1 first: each pointer is one row stride into its array
         constexpr int z = lvl_size(NL, true);
@@ -85,14 +76,8 @@ __device__ __forceinline__ Lv<Real> level_ptrs(Real* arena) {
         return Lv<Real>{b, b + z, b + 2 * z, b + 3 * z, b + 4 * z, b + 5 * z};
     }
     constexpr int z = lvl_size(NL);
-    if constexpr (!CP) {
-        Real* b = arena + lvl_offset(N, NL);
-        return Lv<Real>{b, b + z, b + 2 * z, b + 3 * z, b + 4 * z, b + 5 * z};
-    } else {
-        static_assert(NL < N, "the two-CTA form keeps its top level apart");
-        Real* b = arena + coarse_offset_cp(N / 2, NL);
-        return Lv<Real>{b, b + z, nullptr, b + 2 * z, nullptr, b + 3 * z};
-    }
+    Real* b = arena + lvl_offset(N, NL);
+    return Lv<Real>{b, b + z, b + 2 * z, b + 3 * z, b + 4 * z, b + 5 * z};
 }
 
 // load vector at node n from a table: FP64 values, or (hi, lo) float pairs with hi + lo = b
@@ -230,10 +215,10 @@ __device__ __forceinline__ void restrict_gather(const Real* res, const Lv<Real>&
 
 // zero the boundary rings of e, res, rhs on every level from NL down (interior values are always
 // written before they are read; the rings must read as zero)
-template <typename Real, int N, int NL, int T, bool CP = false, bool FC = false>
+template <typename Real, int N, int NL, int T, bool FC = false>
 __device__ __forceinline__ void zero_rings(Real* arena) {
     constexpr int S = fem_row_stride(NL);
-    const Lv<Real> L = level_ptrs<Real, N, NL, CP, FC>(arena);
+    const Lv<Real> L = level_ptrs<Real, N, NL, FC>(arena);
     if constexpr (FC) {
         // ghost rows -1 and NL + 1 (whole rows), and the Dirichlet columns 0 and NL and the padding
         // column NL + 1 of rows 0 .. NL; rows 0 and NL are unknowns here
@@ -242,16 +227,15 @@ __device__ __forceinline__ void zero_rings(Real* arena) {
                         : ((k - 2 * S) / 3) * S + ((k - 2 * S) % 3 == 0 ? 0 : (k - 2 * S) % 3 == 1 ? NL : NL + 1);
             L.e[n] = L.rhs[n] = L.res[n] = Real(0);
         }
-        if constexpr (NL > 4) zero_rings<Real, N, NL / 2, T, false, true>(arena);
+        if constexpr (NL > 4) zero_rings<Real, N, NL / 2, T, true>(arena);
         return;
     }
     for (int k = threadIdx.x; k < 4 * NL; k += T) {   // rows 0 and NL, then columns 0 and NL
         const int n = k <= NL ? k : k <= 2 * NL + 1 ? NL * S + (k - NL - 1)
                                                      : (1 + ((k - 2 * NL - 2) >> 1)) * S + (((k - 2 * NL - 2) & 1) ? NL : 0);
-        L.e[n] = L.rhs[n] = Real(0);
-        if (L.res) L.res[n] = Real(0);
+        L.e[n] = L.rhs[n] = L.res[n] = Real(0);
     }
-    if constexpr (NL > 2) zero_rings<Real, N, NL / 2, T, CP>(arena);
+    if constexpr (NL > 2) zero_rings<Real, N, NL / 2, T>(arena);
 }
 
 // off-diagonal sum at black node n = (i, j) with its red neighbours read as e + P e_c (P1
@@ -379,28 +363,28 @@ __device__ __forceinline__ void phase_sync() {
 // V(1,1) cycle on a coarse level: reads L.rhs, writes L.e. Levels with at most 4 cells per side
 // (<= 9 unknowns) run inside warp 0 only (T = 32, warp barriers); the caller's next block
 // barrier publishes the result.
-template <typename Real, int N, int NL, int T, bool WARP = false, bool CP = false, bool FC = false>
+template <typename Real, int N, int NL, int T, bool WARP = false, bool FC = false>
 __device__ void vcycle_coarse(Real* arena, const Real* dinv) {
     if constexpr (NL == direct_level<Real, FC>(N)) {
-        dense_solve<Real, NL, T, FC>(level_ptrs<Real, N, NL, CP, FC>(arena), dinv);
+        dense_solve<Real, NL, T, FC>(level_ptrs<Real, N, NL, FC>(arena), dinv);
         phase_sync<WARP>();
     } else if constexpr (!WARP && NL <= 4) {
-        if (threadIdx.x < 32) vcycle_coarse<Real, N, NL, 32, true, CP, FC>(arena, dinv);
+        if (threadIdx.x < 32) vcycle_coarse<Real, N, NL, 32, true, FC>(arena, dinv);
         __syncthreads();
         return;
     } else {
-        Lv<Real> L = level_ptrs<Real, N, NL, CP, FC>(arena);
+        Lv<Real> L = level_ptrs<Real, N, NL, FC>(arena);
         if constexpr (NL == 2) {
             constexpr int n11 = fem_row_stride(2) + 1;           // single interior node (1,1)
             if (threadIdx.x == 0) L.e[n11] = L.rhs[n11] * inv_diag<Real, fem_row_stride(2)>(L, n11);
             phase_sync<WARP>();
         } else {
-            Lv<Real> C = level_ptrs<Real, N, NL / 2, CP, FC>(arena);
+            Lv<Real> C = level_ptrs<Real, N, NL / 2, FC>(arena);
             smooth_color<Real, NL, T, FC>(L, 1);   // red pre-sweep done by the restriction above
             phase_sync<WARP>();
             restrict_red<Real, NL / 2, T, FC>(L, C);
             phase_sync<WARP>();
-            vcycle_coarse<Real, N, NL / 2, T, WARP, CP, FC>(arena, dinv);
+            vcycle_coarse<Real, N, NL / 2, T, WARP, FC>(arena, dinv);
             black_prolong<Real, NL, T, FC>(L, C.e);
             phase_sync<WARP>();
             smooth_color<Real, NL, T, FC>(L, 0);
@@ -463,7 +447,7 @@ __device__ __forceinline__ void coarsen_kappa(const Real* kf, Real* kc) {
 // of the staging area, then recurses
 template <typename Real, int N, int NL, int T, bool FC = false>
 __device__ void setup_levels(Real* arena, Real* stage, bool ping) {
-    Lv<Real> L = level_ptrs<Real, N, NL, false, FC>(arena);
+    Lv<Real> L = level_ptrs<Real, N, NL, FC>(arena);
     Real* kin = ping ? stage : stage + 2 * N * N;
     build_coeffs<Real, NL, T>(L, kin);
     if constexpr (NL > 2) {
@@ -479,27 +463,12 @@ __device__ void setup_levels(Real* arena, Real* stage, bool ping) {
     }
 }
 
-// two-CTA form: coefficients of coarse level NL from kappa in kin, coarser kappa into kout, then
-// recurse with the buffers swapped (no stored inverse diagonal)
-template <typename Real, int N, int NL, int T>
-__device__ void setup_levels_cp(Real* arena, Real* kin, Real* kout) {
-    Lv<Real> L = level_ptrs<Real, N, NL, true>(arena);
-    build_coeffs<Real, NL, T>(L, kin);
-    if constexpr (NL > 2) {
-        coarsen_kappa<Real, NL / 2, T>(kin, kout);
-        __syncthreads();
-        setup_levels_cp<Real, N, NL / 2, T>(arena, kout, kin);
-    } else {
-        __syncthreads();
-    }
-}
-
 // flow cell: the ghost rows -1 and NL + 1 of the coefficient arrays on every level down to 1/4
 // (the boundary rows' stencils read aN there); set before the coefficients are built
 template <typename Real, int N, int NL, int T>
 __device__ __forceinline__ void zero_ghost_weights(Real* arena) {
     constexpr int S = fem_row_stride(NL);
-    const Lv<Real> L = level_ptrs<Real, N, NL, false, true>(arena);
+    const Lv<Real> L = level_ptrs<Real, N, NL, true>(arena);
     for (int k = threadIdx.x; k < 2 * S; k += T) {
         const int n = k < S ? k - S : (NL + 1) * S + (k - S);
         L.aE[n] = L.aN[n] = L.iD[n] = Real(0);
@@ -535,7 +504,7 @@ __device__ __forceinline__ void solve_particle(const FemArgs& a, const int p, Re
     constexpr int E = 2 * N * N;
     const int tid = threadIdx.x;
 
-    Lv<Real> F = level_ptrs<Real, N, N, false, FC>(arena);
+    Lv<Real> F = level_ptrs<Real, N, N, FC>(arena);
     Real* stage = F.e;     // e, res, p of the fine level are contiguous: 3*lvl_size(N) >= 2.5 N^2
     if constexpr (FC) zero_ghost_weights<Real, N, N, T>(arena);   // read by the boundary rows
 
@@ -558,12 +527,12 @@ __device__ __forceinline__ void solve_particle(const FemArgs& a, const int p, Re
 
     // 2) stencil hierarchy
     setup_levels<Real, N, N, T, FC>(arena, stage, true);
-    zero_rings<Real, N, N, T, false, FC>(arena);
+    zero_rings<Real, N, N, T, FC>(arena);
     __syncthreads();
     Real* dinv = arena + arena_size(N, FC) + 4 * NPT * T;
     if constexpr (direct_level<Real, FC>(N) != 0)
         dense_setup<Real, direct_level<Real, FC>(N), T, FC>(
-            level_ptrs<Real, N, direct_level<Real, FC>(N), false, FC>(arena), dinv);
+            level_ptrs<Real, N, direct_level<Real, FC>(N), FC>(arena), dinv);
 
     // fine nodes owned by this thread, one packed int each: bits 0-12 node index n, 13-23 the
     // coarse node c under it ((j/2) SC + i/2), 24-25 (i & 1) + 2 (j & 1), 26 red, 27 valid.
@@ -638,7 +607,7 @@ __device__ __forceinline__ void solve_particle(const FemArgs& a, const int p, Re
     int parity = 0;
     int total_it = 0;
     bool converged = false;
-    Lv<Real> C1 = level_ptrs<Real, N, N / 2, false, FC>(arena);
+    Lv<Real> C1 = level_ptrs<Real, N, N / 2, FC>(arena);
     Real* P = F.rhs;   // fine-level CG direction (the fine rhs is r, held in registers)
 
     for (int pass = 0; pass < a.max_outer && !converged; ++pass) {
@@ -681,7 +650,7 @@ __device__ __forceinline__ void solve_particle(const FemArgs& a, const int p, Re
             __syncthreads();
             restrict_gather<Real, N / 2, T, FC>(F.res, C1);
             __syncthreads();
-            vcycle_coarse<Real, N, N / 2, T, false, false, FC>(arena, dinv);
+            vcycle_coarse<Real, N, N / 2, T, false, FC>(arena, dinv);
 #pragma unroll
             for (int q = NPH; q < NPT; ++q) {
                 z[q] = Real(0);
@@ -846,14 +815,14 @@ __device__ __forceinline__ void solve_particle(const FemArgs& a, const int p, Re
 // arena of a top level N), levels 1/h <= 64 in shared memory (the arena of a top level 64).
 template <typename Real, int N, int NL, bool FC = false>
 __device__ __forceinline__ Lv<Real> ptrs2(Real* garena, Real* sarena) {
-    if constexpr (NL > 64) return level_ptrs<Real, N, NL, false, FC>(garena);
-    else return level_ptrs<Real, 64, NL, false, FC>(sarena);
+    if constexpr (NL > 64) return level_ptrs<Real, N, NL, FC>(garena);
+    else return level_ptrs<Real, 64, NL, FC>(sarena);
 }
 
 template <typename Real, int N, int NL, int T, bool FC = false>
 __device__ void vcycle2(Real* garena, Real* sarena, const Real* dinv) {
     if constexpr (NL <= 64) {
-        vcycle_coarse<Real, 64, NL, T, false, false, FC>(sarena, dinv);
+        vcycle_coarse<Real, 64, NL, T, false, FC>(sarena, dinv);
     } else {
         Lv<Real> L = ptrs2<Real, N, NL, FC>(garena, sarena);
         Lv<Real> C = ptrs2<Real, N, NL / 2, FC>(garena, sarena);
@@ -882,7 +851,7 @@ __device__ __forceinline__ void solve_particle_mem(const FemArgs& a, const int p
     constexpr int E = 2 * N * N;
     constexpr int SC = fem_row_stride(N / 2);
     const int tid = threadIdx.x;
-    Lv<Real> F = level_ptrs<Real, N, N, false, FC>(arena);
+    Lv<Real> F = level_ptrs<Real, N, N, FC>(arena);
     Real* vec = arena + arena_size(N, FC);
     Real *R = vec, *Dv = vec + NI, *XH = vec + 2 * NI, *XL = vec + 3 * NI, *RH = vec + 4 * NI, *RL = vec + 5 * NI;
     // A p is kept in the fine level's residual array (dead outside the restriction): one array
@@ -906,7 +875,7 @@ __device__ __forceinline__ void solve_particle_mem(const FemArgs& a, const int p
         build_diag<Real, N, T, FC>(F);
         Real* k64 = k1;
         if constexpr (N == 256) {
-            Lv<Real> L1 = level_ptrs<Real, N, 128, false, FC>(arena);
+            Lv<Real> L1 = level_ptrs<Real, N, 128, FC>(arena);
             build_coeffs<Real, 128, T>(L1, k1);
             coarsen_kappa<Real, 64, T>(k1, stage);
             __syncthreads();
@@ -934,7 +903,7 @@ __device__ __forceinline__ void solve_particle_mem(const FemArgs& a, const int p
     __syncthreads();
     Real* dinv = sarena + arena_size(64, FC);
     dense_setup<Real, direct_level<Real, FC>(64), T, FC>(
-        level_ptrs<Real, 64, direct_level<Real, FC>(64), false, FC>(sarena), dinv);
+        level_ptrs<Real, 64, direct_level<Real, FC>(64), FC>(sarena), dinv);
     const Real h2 = Real(1) / (Real(N) * Real(N));
     Real bflow = 0;   // flow cell: sum of b^2
     for (int i = tid; i < NI; i += T) {   // r = b: the load vector (h^2 at every node for f = 1)
@@ -1238,462 +1207,6 @@ fem_eval_kernel_fc(FemArgs a) {
                                                    theta_s);
 }
 
-// ---- two-CTA cluster form of the 1/128 solve (mixed path) ------------------------------------
-// One particle per cluster of two CTAs, one CTA per SM. CTA r keeps the fine rows 64 r + 1 ..
-// 64 r + 64 of the 1/128 level on chip (rank 1's last row, 128, is the boundary) with one halo row
-// on either side; the coarse levels 1/64 .. 1/2 are replicated, and both CTAs run the coarse
-// V-cycle on identical data. A value the partner reads (the boundary row of a sweep, the red
-// residuals of row 65, the coarse rows a CTA restricts) is also stored into the partner's shared
-// memory (distributed shared memory), and every fine-level phase ends at a cluster barrier
-// (release / acquire at cluster scope). A reduction sums the 64 warp partials of both CTAs in one
-// fixed order, so both CTAs hold bit-identical scalars and take the same branches: no barrier is
-// left waiting. Fine-level arrays (local index (j - 64 r) S + i, local rows 0 .. 65): edge
-// weights aE, aN; e, which also holds the CG direction p (p is dead while the V-cycle runs and e
-// is dead between the red post-sweep and the next pre-sweep); the red residuals in an array of
-// their own indexed by n / 2. The inverse diagonals are formed from the edge weights where a
-// sweep needs them (approximate reciprocal: they only shape the preconditioner).
-namespace cl {
-constexpr int N = 128, T = 1024, S = fem_row_stride(N), SC = fem_row_stride(N / 2);
-constexpr int FS = 66 * S;                    // floats per strip array (local rows 0 .. 65)
-constexpr int RS = padded(FS / 2);            // red-only residual array
-constexpr int NPT = 8, NPH = 4;               // fine slots per thread (4 red, 4 black)
-constexpr int OFF_AE = 0, OFF_AN = FS, OFF_E = 2 * FS, OFF_RES = 3 * FS, OFF_C = 3 * FS + RS;
-constexpr int OFF_DINV = OFF_C + coarse_size_cp(N / 2);
-constexpr int SMEM_FLOATS = OFF_DINV + dense_reals<float>(N);
-constexpr int REF_FLOATS = 4 * NPT * T;       // refinement state of one CTA (device memory)
-static_assert(fine_slots(N, T) == 2 * NPT, "two CTAs share the fine slots");
-static_assert(OFF_C % 4 == 0 && FS % 4 == 0, "16-byte aligned arrays");
-static_assert(SMEM_FLOATS * 4 <= 227 * 1024, "shared memory of one CTA");
-// packed slot: bits 0-13 local node, 14-26 coarse node under it, 27-28 (i & 1) + 2 (j & 1),
-// 29 red, 30 valid, 31 on the row the partner keeps as its halo
-__device__ __forceinline__ int sn(unsigned s) { return (int)(s & 0x3fffu); }
-__device__ __forceinline__ int sc(unsigned s) { return (int)((s >> 14) & 0x1fffu); }
-__device__ __forceinline__ int scode(unsigned s) { return (int)((s >> 27) & 3u); }
-__device__ __forceinline__ bool sv(unsigned s) { return (s >> 30) & 1u; }
-__device__ __forceinline__ bool ssend(unsigned s) { return (s >> 31) != 0u; }
-}  // namespace cl
-
-__device__ __forceinline__ uint32_t smem_addr(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
-__device__ __forceinline__ int cluster_rank() {
-    uint32_t r;
-    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
-    return (int)r;
-}
-// address of the same shared-memory location in CTA `rank` of the cluster
-__device__ __forceinline__ uint32_t peer_addr(uint32_t a, int rank) {
-    uint32_t r;
-    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(rank));
-    return r;
-}
-__device__ __forceinline__ void st_peer(uint32_t a, float v) {
-    asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(a), "f"(v) : "memory");
-}
-__device__ __forceinline__ void st_peer(uint32_t a, int v) {
-    asm volatile("st.shared::cluster.s32 [%0], %1;" ::"r"(a), "r"(v) : "memory");
-}
-__device__ __forceinline__ float2 ld_peer2(uint32_t a) {
-    float2 v;
-    asm volatile("ld.shared::cluster.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "r"(a) : "memory");
-    return v;
-}
-// all threads of both CTAs; orders shared (local and distributed) and global memory at cluster scope
-__device__ __forceinline__ void cluster_sync() {
-    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
-}
-
-// sum over the cluster: warp sums written to [rank][warp] of both CTAs' buffers, one cluster
-// barrier, then the 64 partials summed in index order (the same value in both CTAs)
-__device__ __forceinline__ float cluster_sum(float a, float* buf, uint32_t peer_buf, int rank) {
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) a += __shfl_xor_sync(0xffffffffu, a, off);
-    if ((threadIdx.x & 31) == 0) {
-        const int k = rank * 32 + (threadIdx.x >> 5);
-        buf[k] = a;
-        st_peer(peer_buf + 4u * k, a);
-    }
-    cluster_sync();
-    float s = 0.f;
-#pragma unroll
-    for (int i = 0; i < 16; ++i) {
-        const float4 v = reinterpret_cast<const float4*>(buf)[i];
-        s += v.x;
-        s += v.y;
-        s += v.z;
-        s += v.w;
-    }
-    return s;
-}
-
-// inverse stencil diagonal at a fine node of the strip, from its four edge weights
-__device__ __forceinline__ float cl_idiag(const float* aE, const float* aN, int n) {
-    return recip_coarse(aE[n] + aE[n - 1] + aN[n] + aN[n - cl::S]);
-}
-
-// the solve of particle p by the calling cluster (all threads of both CTAs call it); sm: this
-// CTA's dynamic shared memory (cl::SMEM_FLOATS), cbuf: [2][64] reduction buffers, ref: this CTA's
-// refinement state in device memory
-template <bool RHS>
-__device__ void solve_particle_cl(const FemArgs& a, const int p, float* sm, float (*cbuf)[64], float* ref,
-                                  const int rank) {
-    using namespace cl;
-    constexpr int E = 2 * N * N, NI = (N - 1) * (N - 1);
-    const int tid = threadIdx.x, partner = rank ^ 1;
-    float* aE = sm + OFF_AE;
-    float* aN = sm + OFF_AN;
-    float* e = sm + OFF_E;   // also the CG direction p and the refinement's correction d
-    float* res = sm + OFF_RES;
-    float* coarse = sm + OFF_C;
-    float* dinv = sm + OFF_DINV;
-    // partner addresses: this CTA's row j sits at local index (j - 64 r) S + i here and at
-    // (j - 64 (1 - r)) S + i in the partner
-    const int shift = rank ? 64 * S : -64 * S;
-    const uint32_t pe = peer_addr(smem_addr(e), partner) + 4u * (uint32_t)shift;
-    const uint32_t pres = peer_addr(smem_addr(res), partner) + 4u * (uint32_t)(shift / 2);
-    const uint32_t pcb[2] = {peer_addr(smem_addr(cbuf[0]), partner), peer_addr(smem_addr(cbuf[1]), partner)};
-    const Lv<float> C1 = level_ptrs<float, N, N / 2, true>(coarse);
-    const uint32_t pc_rhs = peer_addr(smem_addr(C1.rhs), partner), pc_e = peer_addr(smem_addr(C1.e), partner);
-
-    // 1) stencil of the strip (local rows 0 .. 65 = rows 64 r .. 64 r + 65) straight from kappa,
-    //    kappa of 1/64 staged in e, the replicated hierarchy 1/64 .. 1/2, the 1/4 inverse
-    const float* kp = a.kappa + (size_t)p * E;
-    coarsen_kappa<float, N / 2, T>(kp, e);
-    for (int n = tid; n < FS; n += T) {
-        const int lr = n / S, i = n - lr * S, j = 64 * rank + lr;
-        float ae = 0.f, an = 0.f;
-        if (i <= N && j <= N) {
-            if (i < N) {
-                if (j < N) ae += kp[2 * (j * N + i)];
-                if (j > 0) ae += kp[2 * ((j - 1) * N + i) + 1];
-            }
-            if (j < N) {
-                if (i > 0) an += kp[2 * (j * N + i - 1)];
-                if (i < N) an += kp[2 * (j * N + i) + 1];
-            }
-        }
-        aE[n] = 0.5f * ae;
-        aN[n] = 0.5f * an;
-    }
-    __syncthreads();
-    setup_levels_cp<float, N, N / 2, T>(coarse, e, res);
-    for (int n = tid; n < FS + RS; n += T) e[n] = 0.f;   // e and res (contiguous): zero halos and rings
-    zero_rings<float, N, N / 2, T, true>(coarse);
-    if (tid < 32) dense_setup<float, 4, 32>(level_ptrs<float, N, 4, true>(coarse), dinv);
-    cluster_sync();   // also: the partner writes into this CTA's arrays only after they are zeroed
-
-    unsigned slot[NPT];
-    const int send_row = rank ? 65 : 64;
-#pragma unroll
-    for (int q = 0; q < NPT; ++q) {
-        const bool red = q < NPH;
-        int ii, jj;
-        const bool v = colour_node<N>(4096 * rank + tid + T * (red ? q : q - NPH), red ? 0 : 1, ii, jj);
-        if (!v) {
-            ii = 1;
-            jj = 64 * rank + 1;
-        }
-        const unsigned nl = (unsigned)((jj - 64 * rank) * S + ii);
-        const unsigned c = (unsigned)((jj >> 1) * SC + (ii >> 1));
-        const unsigned code = (unsigned)((ii & 1) + 2 * (jj & 1));
-        slot[q] = nl | (c << 14) | (code << 27) | ((red ? 1u : 0u) << 29) | ((v ? 1u : 0u) << 30) |
-                  ((v && jj == send_row) ? 1u : 0u) << 31;
-    }
-    const float h2 = 1.f / (float(N) * float(N));
-    auto XH = [&](int q) -> float& { return ref[(0 * NPT + q) * T + tid]; };
-    auto XL = [&](int q) -> float& { return ref[(1 * NPT + q) * T + tid]; };
-    auto RH = [&](int q) -> float& { return ref[(2 * NPT + q) * T + tid]; };
-    auto RL = [&](int q) -> float& { return ref[(3 * NPT + q) * T + tid]; };
-#pragma unroll
-    for (int q = 0; q < NPT; ++q) {
-        XH(q) = XL(q) = RL(q) = 0.f;
-        RH(q) = sv(slot[q]) ? h2 : 0.f;
-    }
-    if (RHS && a.rhs) {
-#pragma unroll 1
-        for (int q = 0; q < NPT; ++q) {
-            const bool red = q < NPH;
-            int ii, jj;
-            if (colour_node<N>(4096 * rank + tid + T * (red ? q : q - NPH), red ? 0 : 1, ii, jj)) {
-                float hi, lo;
-                load_rhs(a.rhs, jj * S + ii, hi, lo);
-                RH(q) = hi;
-                RL(q) = lo;
-            }
-        }
-    }
-    float r[NPT], d[NPT], z[NPT], pv[NPT];
-    const float bnorm2 = (RHS && a.rhs) ? float(a.bnorm2) : float(NI) * h2 * h2;
-    const float stop_outer = float(a.rtol * a.rtol) * bnorm2;
-    const float stop_last = float(0.25 * a.rtol * a.rtol) * bnorm2;
-    const float rtol_in2 = float(a.rtol_in * a.rtol_in);
-    int parity = 0, total_it = 0;
-    bool converged = false;
-    // coarse rows this CTA restricts: 1 .. 32 (rank 0; row 32 reads the red residuals of row 65
-    // from the halo) or 33 .. 63 (rank 1)
-    const int J0 = rank ? 33 : 1, NJ = rank ? 31 : 32;
-
-    for (int pass = 0; pass < a.max_outer && !converged; ++pass) {
-        float rr0 = 0.f;
-#pragma unroll
-        for (int q = 0; q < NPT; ++q) {
-            r[q] = RH(q);
-            d[q] = 0.f;
-            pv[q] = 0.f;
-            rr0 += r[q] * r[q];
-        }
-#pragma unroll
-        for (int q = 0; q < NPH; ++q)   // red pre-sweep of the first cycle
-            if (sv(slot[q])) {
-                const int n = sn(slot[q]);
-                const float v = r[q] * cl_idiag(aE, aN, n);
-                e[n] = v;
-                if (ssend(slot[q])) st_peer(pe + 4u * n, v);
-            }
-        rr0 = cluster_sum(rr0, cbuf[parity], pcb[parity], rank);
-        parity ^= 1;
-        if (!(rr0 > 0.f)) break;
-        const float stop2 = fmaxf(rtol_in2 * rr0, stop_last);
-        float rz = 0.f;
-        for (int it = 0; it < a.max_inner; ++it) {
-            // black pre-sweep
-#pragma unroll
-            for (int q = NPH; q < NPT; ++q)
-                if (sv(slot[q])) {
-                    const int n = sn(slot[q]);
-                    const float v = (r[q] + offsum<float, S>(aE, aN, e, n)) * cl_idiag(aE, aN, n);
-                    e[n] = v;
-                    if (ssend(slot[q])) st_peer(pe + 4u * n, v);
-                }
-            cluster_sync();
-            // red residuals (rank 1 also sends row 65, which rank 0 restricts into coarse row 32)
-#pragma unroll
-            for (int q = 0; q < NPH; ++q)
-                if (sv(slot[q])) {
-                    const int n = sn(slot[q]);
-                    const float v = offsum<float, S>(aE, aN, e, n);
-                    res[n >> 1] = v;
-                    if (rank == 1 && ssend(slot[q])) st_peer(pres + 4u * (n >> 1), v);
-                }
-            cluster_sync();
-            // restriction of this CTA's coarse rows into both CTAs (with the coarse red pre-sweep)
-            for (int idx = tid; idx < NJ * (N / 2 - 1); idx += T) {
-                const int Jr = idx / (N / 2 - 1), J = J0 + Jr, I = idx - Jr * (N / 2 - 1) + 1;
-                const int f = (2 * J - 64 * rank) * S + 2 * I, c = J * SC + I;
-                const float v = res[f >> 1] + 0.5f * (res[(f + S + 1) >> 1] + res[(f - S - 1) >> 1]);
-                C1.rhs[c] = v;
-                st_peer(pc_rhs + 4u * c, v);
-                if (((I + J) & 1) == 0) {
-                    const float ev = v * inv_diag<float, SC>(C1, c);
-                    C1.e[c] = ev;
-                    st_peer(pc_e + 4u * c, ev);
-                }
-            }
-            cluster_sync();
-            vcycle_coarse<float, N, N / 2, T, false, true>(coarse, dinv);
-            // black post-sweep with the prolongation folded in
-#pragma unroll
-            for (int q = NPH; q < NPT; ++q) {
-                z[q] = 0.f;
-                if (sv(slot[q])) {
-                    const int n = sn(slot[q]);
-                    const float v = (r[q] + offsum_prolong<float, S, SC>(aE, aN, e, C1.e, n, sc(slot[q]),
-                                                                          scode(slot[q]) == 1)) *
-                                    cl_idiag(aE, aN, n);
-                    z[q] = v;
-                    e[n] = v;
-                    if (ssend(slot[q])) st_peer(pe + 4u * n, v);
-                }
-            }
-            cluster_sync();
-            float rz_new = 0.f;
-#pragma unroll
-            for (int q = 0; q < NPH; ++q) {   // red post-sweep
-                z[q] = 0.f;
-                if (sv(slot[q])) {
-                    const int n = sn(slot[q]);
-                    z[q] = (r[q] + offsum<float, S>(aE, aN, e, n)) * cl_idiag(aE, aN, n);
-                }
-            }
-#pragma unroll
-            for (int q = 0; q < NPT; ++q) rz_new += r[q] * z[q];
-            rz_new = cluster_sum(rz_new, cbuf[parity], pcb[parity], rank);
-            parity ^= 1;
-            const float beta = (it == 0) ? 0.f : rz_new / rz;
-            rz = rz_new;
-#pragma unroll
-            for (int q = 0; q < NPT; ++q) {
-                pv[q] = (it == 0) ? z[q] : z[q] + beta * pv[q];
-                if (sv(slot[q])) {
-                    e[sn(slot[q])] = pv[q];
-                    if (ssend(slot[q])) st_peer(pe + 4u * sn(slot[q]), pv[q]);
-                }
-            }
-            cluster_sync();
-            float qv[NPT];
-            float pq = 0.f;
-#pragma unroll
-            for (int q = 0; q < NPT; ++q) {
-                qv[q] = 0.f;
-                if (sv(slot[q])) {
-                    qv[q] = stencil_apply_at<float, S>(aE, aN, e, sn(slot[q]), pv[q]);
-                    pq += pv[q] * qv[q];
-                }
-            }
-            pq = cluster_sum(pq, cbuf[parity], pcb[parity], rank);
-            parity ^= 1;
-            const float alpha = rz / pq;
-            float rr = 0.f;
-#pragma unroll
-            for (int q = 0; q < NPT; ++q) {
-                d[q] = fmaf(alpha, pv[q], d[q]);
-                r[q] = fmaf(-alpha, qv[q], r[q]);
-                rr += r[q] * r[q];
-            }
-#pragma unroll
-            for (int q = 0; q < NPH; ++q)   // red pre-sweep of the next cycle
-                if (sv(slot[q])) {
-                    const int n = sn(slot[q]);
-                    const float v = r[q] * cl_idiag(aE, aN, n);
-                    e[n] = v;
-                    if (ssend(slot[q])) st_peer(pe + 4u * n, v);
-                }
-            rr = cluster_sum(rr, cbuf[parity], pcb[parity], rank);
-            parity ^= 1;
-            ++total_it;
-            if (!(rr > stop2)) break;
-        }
-        // refinement: x += d, r -= A d in double-float arithmetic (edge form, as in the one-CTA forms)
-#pragma unroll
-        for (int q = 0; q < NPT; ++q)
-            if (sv(slot[q])) {
-                e[sn(slot[q])] = d[q];
-                if (ssend(slot[q])) st_peer(pe + 4u * sn(slot[q]), d[q]);
-            }
-        cluster_sync();
-        float rr_out = 0.f;
-#pragma unroll
-        for (int q = 0; q < NPT; ++q)
-            if (sv(slot[q])) {
-                const int n = sn(slot[q]);
-                const float di = e[n];
-                const float w[4] = {aE[n], aE[n - 1], aN[n], aN[n - S]};
-                const float dj[4] = {e[n + 1], e[n - 1], e[n + S], e[n - S]};
-                float ah = 0.f, al = 0.f;
-#pragma unroll
-                for (int t = 0; t < 4; ++t) {
-                    float sh, sl;
-                    two_sum(di, -dj[t], sh, sl);
-                    const float ph = __fmul_rn(w[t], sh);
-                    float pl = fmaf(w[t], sh, -ph);
-                    pl = fmaf(w[t], sl, pl);
-                    df_add(ah, al, ph, pl);
-                }
-                float rh = RH(q), rl = RL(q), xh = XH(q), xl = XL(q);
-                df_add(rh, rl, -ah, -al);
-                df_add(xh, xl, d[q], 0.f);
-                RH(q) = rh;
-                RL(q) = rl;
-                XH(q) = xh;
-                XL(q) = xl;
-                rr_out += rh * rh;
-            }
-        rr_out = cluster_sum(rr_out, cbuf[parity], pcb[parity], rank);
-        parity ^= 1;
-        converged = rr_out <= stop_outer;
-    }
-
-    // ---- observations and misfit (FP64): each CTA writes its strip's solution (double-float pair
-    // as float2, boundary nodes zero) over the edge weights; warp 0 of rank 0 gathers from both
-    float2* xs = reinterpret_cast<float2*>(aE);   // FS float2 = the aE and aN arrays
-    for (int n = tid; n < FS; n += T) xs[n] = make_float2(0.f, 0.f);
-    __syncthreads();
-#pragma unroll
-    for (int q = 0; q < NPT; ++q)
-        if (sv(slot[q])) xs[sn(slot[q])] = make_float2(XH(q), XL(q));
-    cluster_sync();
-    if (rank == 0 && tid < 32) {
-        const uint32_t pxs = peer_addr(smem_addr(xs), 1);
-        auto val = [&](int n) -> double {   // n = j S + i on the whole level
-            const int j = n / S, i = n - j * S;
-            float2 v;
-            if (j <= 64) v = xs[j * S + i];
-            else v = ld_peer2(pxs + 8u * (uint32_t)((j - 64) * S + i));
-            return (double)v.x + (double)v.y;
-        };
-        double misfit = 0.0;
-        for (int o = tid; o < a.n_obs; o += 32) {
-            const double g = a.obs_w[3 * o] * val(a.obs_idx[3 * o]) + a.obs_w[3 * o + 1] * val(a.obs_idx[3 * o + 1]) +
-                             a.obs_w[3 * o + 2] * val(a.obs_idx[3 * o + 2]);
-            if (a.G) a.G[(size_t)p * a.n_obs + o] = g;
-            const double rdf = a.y[o] - g;
-            misfit += rdf * rdf;
-        }
-#pragma unroll
-        for (int off = 16; off > 0; off >>= 1) misfit += __shfl_xor_sync(0xffffffffu, misfit, off);
-        if (tid == 0) {
-            a.Phi[p] = 0.5 * misfit * a.inv_sigma2;
-            if (a.iters) a.iters[p] = converged ? total_it : -(total_it + 1);
-        }
-    }
-}
-
-// persistent clusters: rank 0 takes the next particle from the counter and hands it to rank 1;
-// the cluster barrier at the end of each particle keeps either CTA from overwriting memory the
-// other still reads (halo rows, coarse rows, the solution gathered by rank 0, the ticket)
-template <bool RHS>
-__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(cl::T, 1)
-    fem_eval_cluster(FemArgs a, float* ref_scratch, int* counter) {
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    __shared__ __align__(16) float cbuf[2][64];
-    __shared__ int item_s;
-    const int rank = cluster_rank();
-    float* ref = ref_scratch + (size_t)blockIdx.x * cl::REF_FLOATS;
-    const uint32_t p_item = peer_addr(smem_addr(&item_s), rank ^ 1);
-    for (;;) {
-        if (rank == 0 && threadIdx.x == 0) {
-            const int item = atomicAdd(counter, 1);
-            item_s = item;
-            st_peer(p_item, item);
-        }
-        cluster_sync();
-        const int item = item_s;
-        if (item >= a.n) break;   // the same item in both CTAs
-        solve_particle_cl<RHS>(a, item, reinterpret_cast<float*>(smem_raw), cbuf, ref, rank);
-        cluster_sync();
-    }
-}
-
-// many problems at 1/128: the same persistent clusters take (problem, particle) items; the item's
-// problem is found in a per-item table and each CTA copies its launch arguments to shared memory
-__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(cl::T, 1)
-    fem_eval_cluster_multi(const FemArgs* groups, const int* offsets, const int* item_group, int total,
-                           float* ref_scratch, int* counter) {
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    __shared__ __align__(16) float cbuf[2][64];
-    __shared__ int item_s, p_s;
-    __shared__ FemArgs args_s;
-    const int rank = cluster_rank();
-    float* ref = ref_scratch + (size_t)blockIdx.x * cl::REF_FLOATS;
-    const uint32_t p_item = peer_addr(smem_addr(&item_s), rank ^ 1);
-    for (;;) {
-        if (rank == 0 && threadIdx.x == 0) {
-            const int item = atomicAdd(counter, 1);
-            item_s = item;
-            st_peer(p_item, item);
-        }
-        cluster_sync();
-        const int item = item_s;
-        if (item >= total) break;   // the same item in both CTAs
-        if (threadIdx.x == 0) {
-            const int g = item_group[item];
-            args_s = groups[g];
-            p_s = item - offsets[g];
-        }
-        __syncthreads();
-        solve_particle_cl<true>(args_s, p_s, reinterpret_cast<float*>(smem_raw), cbuf, ref, rank);
-        cluster_sync();
-    }
-}
-
 // persistent form: grid-sized blocks pull (group, particle) items from a device counter; every
 // group is one problem's launch arguments at this level size (many independent inverse problems
 // in one launch)
@@ -1791,56 +1304,7 @@ cudaError_t launch_global_multi(const FemArgs* groups, const int* offsets, const
     return cudaGetLastError();
 }
 
-// ---- two-CTA cluster form of 1/128 ----
-template <bool RHS>
-int cluster_resident_clusters() {
-    const size_t smem = sizeof(float) * (size_t)cl::SMEM_FLOATS;
-    cudaFuncSetAttribute(fem_eval_cluster<RHS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(2, 1, 1);
-    cfg.blockDim = dim3(cl::T, 1, 1);
-    cfg.dynamicSmemBytes = smem;
-    int n = 0;
-    if (cudaOccupancyMaxActiveClusters(&n, (const void*)fem_eval_cluster<RHS>, &cfg) != cudaSuccess) {
-        cudaGetLastError();
-        return 0;
-    }
-    return n;
-}
-
-template <bool RHS>
-cudaError_t launch_cluster_t(const FemArgs& a, float* ref_scratch, int blocks, int* counter, cudaStream_t st) {
-    const size_t smem = sizeof(float) * (size_t)cl::SMEM_FLOATS;
-    cudaError_t e = cudaFuncSetAttribute(fem_eval_cluster<RHS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    fem_eval_cluster<RHS><<<blocks, cl::T, smem, st>>>(a, ref_scratch, counter);
-    count_launches(1);
-    return cudaGetLastError();
-}
-
 }  // namespace
-
-int fem_cluster_blocks() {
-    // CTAs of the two-CTA form that are resident at once, queried once per device
-    static int cached[64] = {};
-    int dev = 0;
-    cudaGetDevice(&dev);
-    if (dev >= 0 && dev < 64 && cached[dev] > 0) return cached[dev];
-    const int blocks = 2 * cluster_resident_clusters<false>();
-    if (dev >= 0 && dev < 64 && blocks > 0) cached[dev] = blocks;
-    return blocks;
-}
-size_t fem_cluster_ref_floats() { return (size_t)cl::REF_FLOATS; }
-
-cudaError_t fem_eval_cluster_launch(const FemArgs& a, float* ref_scratch, int blocks, int* counter, cudaStream_t st) {
-    if (a.n <= 0) return cudaSuccess;
-    if (a.N != 128 || a.precision != SMC_MIXED || !a.kappa || a.flow_cell || blocks < 2) return cudaErrorInvalidValue;
-    const int grid = 2 * std::max(1, std::min(a.n, blocks / 2));
-    cudaError_t e = cudaMemsetAsync(counter, 0, sizeof(int), st);
-    if (e != cudaSuccess) return e;
-    return a.rhs ? launch_cluster_t<true>(a, ref_scratch, grid, counter, st)
-                 : launch_cluster_t<false>(a, ref_scratch, grid, counter, st);
-}
 
 size_t fem_global_slice(int N, bool FC) {
     const int NI = (N - 1) * (FC ? N + 1 : N - 1);
@@ -1879,33 +1343,9 @@ cudaError_t fem_eval_global_launch(const FemArgs& a, float* scratch, int blocks,
     return cudaErrorInvalidValue;
 }
 
-bool fem_cluster_form(int N, int precision, bool flow_cell) {
-    return N == 128 && precision == SMC_MIXED && !flow_cell && fem_cluster_blocks() >= 2;
-}
-
-size_t fem_large_multi_scratch(int N) {
-    if (fem_cluster_form(N, SMC_MIXED, false)) return (size_t)fem_cluster_blocks() * cl::REF_FLOATS;
-    return (size_t)fem_global_blocks(N) * fem_global_slice(N);
-}
-
 size_t fem_multi_scratch(int N, int precision) {
-    if (N >= 128) return fem_large_multi_scratch(N);
-    return fem_tile_form(N, precision, false) ? fem_tile_scratch(N) : 0;
-}
-
-cudaError_t fem_eval_large_multi_launch(int N, const FemArgs* groups, const int* offsets, const int* item_group,
-                                        int total, float* scratch, int* counter, cudaStream_t st) {
-    if (total <= 0) return cudaSuccess;
-    if (!fem_cluster_form(N, SMC_MIXED, false))
-        return fem_eval_global_multi_launch(N, groups, offsets, item_group, total, scratch, fem_global_blocks(N),
-                                            counter, st);
-    const size_t smem = sizeof(float) * (size_t)cl::SMEM_FLOATS;
-    cudaError_t e = cudaFuncSetAttribute(fem_eval_cluster_multi, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    const int grid = 2 * std::max(1, std::min(total, fem_cluster_blocks() / 2));
-    fem_eval_cluster_multi<<<grid, cl::T, smem, st>>>(groups, offsets, item_group, total, scratch, counter);
-    count_launches(1);
-    return cudaGetLastError();
+    if (fem_tile_form(N, precision, false)) return fem_tile_scratch(N);
+    return N >= 128 ? (size_t)fem_global_blocks(N) * fem_global_slice(N) : 0;
 }
 
 cudaError_t fem_eval_global_multi_launch(int N, const FemArgs* groups, const int* offsets, const int* item_group,
@@ -1952,9 +1392,8 @@ bool fem_level_supported(int N, int precision) {
 // -256 on 1/64 and 1/32, where every size names the register-tiled form (fem_tile.cu)
 int fem_default_block(int N, int precision) {
     if (precision == SMC_MIXED && (N == 32 || N == 64)) return N == 64 ? -512 : -256;
-    // 1/128: the two-CTA cluster form where a cluster fits (1.2x the device-memory form at J = 4000
-    // and 8000), else the device-memory form
-    if (precision == SMC_MIXED && N == 128) return fem_cluster_blocks() >= 2 ? -1024 : 1024;
+    // 1/128: the two-CTA cluster form where a cluster fits, else the device-memory form
+    if (precision == SMC_MIXED && N == 128) return fem_tile_form(N, precision, false) ? -1024 : 1024;
     const std::vector<int> s = fem_block_sizes(N, precision);
     return s.empty() ? 0 : s[0];
 }

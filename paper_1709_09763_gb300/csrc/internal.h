@@ -85,30 +85,15 @@ cudaError_t fem_eval_global_multi_launch(int N, const FemArgs* groups, const int
 // items to the blocks
 cudaError_t fem_eval_persistent_launch(int N, int precision, int T, const FemArgs* groups, const int* offsets,
                                        const int* item_group, int total, int* counter, cudaStream_t st);
-// register-tiled form of the mixed Dirichlet solve on 1/64 and 1/32 (fem_tile.cu), every block size of
-// those levels: persistent blocks (2 of 256 threads an SM on 1/64, 8 of 64 on 1/32) with
-// fem_tile_scratch(N) floats of device scratch for their refinement state. *counter (device) is
-// reset by fem_tile_launch; fem_tile_multi_launch (arguments as fem_eval_persistent_launch) needs it
-// zero
+// register-tiled form of the mixed solve (fem_tile.cu): 1/32 and 1/64 on one CTA (every block size of those
+// levels), 1/128 on a cluster of two CTAs (block size -1024), 1/256 of eight; not the flow cell. Where a
+// cluster does not fit, 1/128 and 1/256 run in the device-memory form above. fem_tile_scratch floats of device scratch hold the refinement state. *counter (device) is reset by
+// fem_tile_launch; fem_tile_multi_launch (arguments as fem_eval_persistent_launch) needs it zero
 bool fem_tile_form(int N, int precision, bool flow_cell);
 size_t fem_tile_scratch(int N);
 cudaError_t fem_tile_launch(const FemArgs& a, float* scratch, int* counter, cudaStream_t st);
 cudaError_t fem_tile_multi_launch(int N, const FemArgs* groups, const int* offsets, const int* item_group, int total,
                                   float* scratch, int* counter, cudaStream_t st);
-// two-CTA cluster form of the mixed 1/128 solve (block size -1024 of fem_block_sizes): the fine
-// level split in row strips over the two CTAs of a cluster, each on its own SM;
-// fem_cluster_blocks() CTAs (0 where no cluster fits) with fem_cluster_ref_floats() floats of
-// device scratch each for the refinement state; *counter (device) is reset by the launch
-int fem_cluster_blocks();
-size_t fem_cluster_ref_floats();
-cudaError_t fem_eval_cluster_launch(const FemArgs& a, float* ref_scratch, int blocks, int* counter, cudaStream_t st);
-// large levels of many problems in the form single solves default to: the two-CTA form on 1/128
-// (mixed, not the flow cell) where a cluster fits, else the device-memory form; scratch floats it
-// needs (sized before any graph capture) and the launch (*counter zero before it)
-bool fem_cluster_form(int N, int precision, bool flow_cell);
-size_t fem_large_multi_scratch(int N);
-cudaError_t fem_eval_large_multi_launch(int N, const FemArgs* groups, const int* offsets, const int* item_group,
-                                        int total, float* scratch, int* counter, cudaStream_t st);
 // device scratch (floats) of a many-problem launch on level N: the large levels', the tile form's, else 0
 size_t fem_multi_scratch(int N, int precision);
 bool fem_level_supported(int N, int precision);
