@@ -94,6 +94,15 @@ __global__ void sample_indices_kernel(int* idx, int B, int count, uint32_t step,
     idx[b] = (int)(((uint64_t)x.x * (uint64_t)count) >> 32);
 }
 
+// standardised targets of B rows of observations (gradient entry point), padded with 0: the arithmetic of
+// batch_kernel
+__global__ void targets_kernel(const double* G, int B, int n_obs, int NOp, const float* mu, const float* sd, float* tgt) {
+    const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    if (t >= (long long)B * NOp) return;
+    const int b = (int)(t / NOp), c = (int)(t - (long long)b * NOp);
+    tgt[t] = c < n_obs ? (float)((G[(size_t)b * n_obs + c] - (double)mu[c]) / (double)sd[c]) : 0.0f;
+}
+
 // dZ = 2 (Z - z) / (B n_obs) on real outputs, 0 on padding; bf16 row-major and transposed;
 // per-block partial sums of squared errors
 __global__ void loss_grad_kernel(const float* Z, const float* tgt, int B, int NOp, int n_obs, __nv_bfloat16* dZ,
@@ -293,13 +302,19 @@ int Handle::mlp_setup(int level) {
         A((void**)&S.Wm[l], n * 4);
         A((void**)&S.mW[l], n * 4);
         A((void**)&S.vW[l], n * 4);
-        A((void**)&S.gW[l], n * 4);
         A((void**)&S.W[l], n * 2);
         A((void**)&S.Wt[l], n * 2);
         A((void**)&S.bm[l], (size_t)S.d[l + 1] * 4);
         A((void**)&S.mb[l], (size_t)S.d[l + 1] * 4);
         A((void**)&S.vb[l], (size_t)S.d[l + 1] * 4);
-        A((void**)&S.gb[l], (size_t)S.d[l + 1] * 4);
+    }
+    // gradients in one allocation, in the order of the flat parameter arrays (every size a multiple of 16)
+    size_t n_grad = 0;
+    for (int l = 0; l < 5; ++l) n_grad += (size_t)S.d[l + 1] * S.d[l] + S.d[l + 1];
+    A((void**)&S.gW[0], n_grad * 4);
+    for (int l = 0; l < 5 && e == cudaSuccess; ++l) {
+        S.gb[l] = S.gW[l] + (size_t)S.d[l + 1] * S.d[l];
+        if (l < 4) S.gW[l + 1] = S.gb[l] + S.d[l + 1];
     }
     A((void**)&S.mu, (size_t)S.d[5] * 4);
     A((void**)&S.sd, (size_t)S.d[5] * 4);
@@ -364,6 +379,7 @@ int Handle::mlp_work(int B) {
     A((void**)&mwork.Z, (size_t)B * dmax * 4);
     A((void**)&mwork.tgt, (size_t)B * dmax * 4);
     A((void**)&mwork.th, (size_t)B * K * 8);
+    A((void**)&mwork.obs, (size_t)B * n_obs * 8);
     A((void**)&mwork.idx, (size_t)B * 4);
     A((void**)&mwork.partial, (size_t)grid_of((long long)B * dmax, 256) * 8);
     // up to 64 split-K slices of a dmax x dmax weight gradient
@@ -385,18 +401,19 @@ void MlpWork::release() {
     for (auto& p : pre) { cudaFree(p); p = nullptr; }
     for (auto& p : dZ) { cudaFree(p); p = nullptr; }
     for (auto& p : dZt) { cudaFree(p); p = nullptr; }
-    cudaFree(Z); cudaFree(tgt); cudaFree(th); cudaFree(idx); cudaFree(partial); cudaFree(splitk);
-    Z = tgt = nullptr; th = nullptr; idx = nullptr; partial = nullptr; splitk = nullptr;
+    cudaFree(Z); cudaFree(tgt); cudaFree(th); cudaFree(obs); cudaFree(idx); cudaFree(partial); cudaFree(splitk);
+    Z = tgt = nullptr; th = obs = nullptr; idx = nullptr; partial = nullptr; splitk = nullptr;
     splitk_floats = 0;
     cap = 0;
 }
 
 void Mlp::release() {
     for (int l = 0; l < 5; ++l) {
-        for (void* p : {(void*)Wm[l], (void*)mW[l], (void*)vW[l], (void*)gW[l], (void*)W[l], (void*)Wt[l],
-                        (void*)bm[l], (void*)mb[l], (void*)vb[l], (void*)gb[l]})
+        for (void* p : {(void*)Wm[l], (void*)mW[l], (void*)vW[l], (void*)W[l], (void*)Wt[l], (void*)bm[l], (void*)mb[l],
+                        (void*)vb[l]})
             cudaFree(p);
     }
+    cudaFree(gW[0]);   // the one allocation behind gW and gb
     cudaFree(mu); cudaFree(sd); cudaFree(ring_th); cudaFree(ring_G); cudaFree(err);
 }
 
@@ -692,27 +709,19 @@ int smc_surrogate_grads(smc_handle* hh, int level, int n, const double* theta, c
     Mlp& S = h->mlps[level];
     rc = h->mlp_work(n);
     if (rc != SMC_OK) return rc;
-    // standardised targets computed on the host side of this test entry point from the set mu, sd
-    std::vector<float> musd((size_t)2 * S.d[5]);
-    cudaMemcpy(musd.data(), S.mu, (size_t)S.d[5] * 4, cudaMemcpyDeviceToHost);
-    cudaMemcpy(musd.data() + S.d[5], S.sd, (size_t)S.d[5] * 4, cudaMemcpyDeviceToHost);
-    std::vector<float> tgt((size_t)n * S.d[5], 0.0f);
-    for (int i = 0; i < n; ++i)
-        for (int o = 0; o < h->n_obs; ++o)
-            tgt[(size_t)i * S.d[5] + o] = (float)((G[(size_t)i * h->n_obs + o] - musd[o]) / musd[S.d[5] + o]);
     cudaError_t e = cudaMemcpyAsync(h->mwork.th, theta, (size_t)n * h->K * 8, cudaMemcpyHostToDevice, h->stream);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(h->mwork.tgt, tgt.data(), tgt.size() * 4, cudaMemcpyHostToDevice, h->stream);
+    if (e == cudaSuccess)
+        e = cudaMemcpyAsync(h->mwork.obs, G, (size_t)n * h->n_obs * 8, cudaMemcpyHostToDevice, h->stream);
     if (e != cudaSuccess) return h->cuda_fail(e, "stage gradient inputs");
+    targets_kernel<<<grid_of((long long)n * S.d[5], 256), 256, 0, h->stream>>>(h->mwork.obs, n, h->n_obs, S.d[5], S.mu,
+                                                                             S.sd, h->mwork.tgt);
+    count_launches(1);
     rc = h->mlp_backward(level, n, loss);
     if (rc != SMC_OK) return rc;
-    size_t off = 0;
-    for (int l = 0; l < 5 && e == cudaSuccess; ++l) {
-        const size_t nw = (size_t)S.d[l + 1] * S.d[l], nb = (size_t)S.d[l + 1];
-        e = cudaMemcpyAsync(grads + off, S.gW[l], nw * 4, cudaMemcpyDeviceToHost, h->stream);
-        off += nw;
-        if (e == cudaSuccess) e = cudaMemcpyAsync(grads + off, S.gb[l], nb * 4, cudaMemcpyDeviceToHost, h->stream);
-        off += nb;
-    }
+    // the ten gradient tensors lie one after the other in the flat order: one copy
+    size_t count = 0;
+    for (int l = 0; l < 5; ++l) count += (size_t)S.d[l + 1] * S.d[l] + S.d[l + 1];
+    e = cudaMemcpyAsync(grads, S.gW[0], count * 4, cudaMemcpyDeviceToHost, h->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
     if (e != cudaSuccess) return h->cuda_fail(e, "copy gradients");
     return SMC_OK;

@@ -20,7 +20,7 @@ struct Mlp {
     int t = 0;                               // Adam steps taken
     float *Wm[5] = {}, *bm[5] = {};          // FP32 master weights
     float *mW[5] = {}, *vW[5] = {}, *mb[5] = {}, *vb[5] = {};
-    float *gW[5] = {}, *gb[5] = {};
+    float *gW[5] = {}, *gb[5] = {};          // one allocation (gW[0]), in the flat parameter order
     __nv_bfloat16 *W[5] = {}, *Wt[5] = {};   // BF16 copies [out][in] and [in][out]
     float *mu = nullptr, *sd = nullptr;      // standardisation of the targets
     double *ring_th = nullptr, *ring_G = nullptr;   // training pairs (theta, G_l(theta))
@@ -35,7 +35,7 @@ struct MlpWork {
     float* pre[5] = {};
     __nv_bfloat16 *dZ[5] = {}, *dZt[5] = {};
     float *Z = nullptr, *tgt = nullptr;
-    double* th = nullptr;
+    double *th = nullptr, *obs = nullptr;
     int* idx = nullptr;
     double* partial = nullptr;
     float* splitk = nullptr;                 // split-K partial tiles of the weight gradients
