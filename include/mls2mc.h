@@ -186,8 +186,8 @@ int smc_set_timing(smc_handle* h, int enable);
  * sizes, best_ms [n_levels] the time per launch (either may be NULL). smc_set_block_size forces a
  * block size for a level (T = 0 restores the default: -512 and -256 on 1/64 and 1/32 of the mixed
  * path, the two-CTA form on 1/128, else the first compiled size); T must be one of the
- * compiled sizes. On 1/64 (512, 1024, -512) and 1/32 (256, 512, -256) of the mixed path every size
- * compiled sizes. On 1/64 (512, 1024, -512) and 1/32 (256, 512, -256) of the mixed path every size
+ * compiled sizes (FP64: 64 at 1/8 runs 32 threads, 256 at 1/32 runs 128). On 1/64 (512, 1024, -512)
+ * and 1/32 (256, 512, -256) of the mixed path every size
  * names the same register-tiled form (two particles per SM on 1/64, eight on 1/32; the flow cell has one
  * form per level of its own). At 1/h = 128, -1024 selects the two-CTA form: one particle per cluster of
  * two CTAs of 512 threads on two SMs, each with half of the two finest levels on chip, border rows

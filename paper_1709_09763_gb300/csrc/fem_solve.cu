@@ -135,6 +135,36 @@ __device__ __forceinline__ void block_sum(Acc& a, double* buf_raw) {
     a = s;
 }
 
+// Sum over the block (into a) and a quotient with it: sum / other (sum_over) or other / sum. On the FP64 path one
+// warp adds the warps' sums and divides for the others -- another one in every block, so that the blocks of an
+// SM spread this over the four schedulers' FP64 units -- because ~14 FP64 instructions in each warp cost more
+// than the second barrier (a 64-cycle slot each, a sixth of an iteration's FP64 time on 1/16).
+template <int T, typename Acc>
+__device__ __forceinline__ Acc block_sum_div(Acc& a, Acc other, bool sum_over, double* buf_raw) {
+    if constexpr (sizeof(Acc) == 4 || T == 32) {
+        block_sum<T>(a, buf_raw);
+        return sum_over ? a / other : other / a;
+    } else {
+#pragma unroll
+        for (int off = 16; off > 0; off >>= 1) a += __shfl_xor_sync(0xffffffffu, a, off);
+        if ((threadIdx.x & 31) == 0) buf_raw[threadIdx.x >> 5] = a;
+        __syncthreads();
+        if ((threadIdx.x >> 5) == (blockIdx.x & (T / 32 - 1))) {
+            double s = 0;
+#pragma unroll
+            for (int i = 0; i < T / 32; ++i) s += buf_raw[i];
+            const double q = sum_over ? s / other : other / s;
+            if ((threadIdx.x & 31) == 0) {
+                buf_raw[32] = s;
+                buf_raw[33] = q;
+            }
+        }
+        __syncthreads();
+        a = buf_raw[32];
+        return buf_raw[33];
+    }
+}
+
 // ---- red/black enumeration -----------------------------------------------------------------
 // Position k of colour col (0 red: i + j even, 1 black) on a level with NL cells per side. A
 // colour has NL/2 positions per row (the last one idle in rows with NL/2 - 1 nodes of that
@@ -274,13 +304,15 @@ __device__ __forceinline__ void black_prolong(const Lv<Real>& L, const Real* ec)
 // m = (NL - 1)^2 = 9 unknowns) is inverted once per particle and applied as a dense
 // matrix-vector product, replacing the cycles of the levels below it. (An exact solve one level
 // higher, m = 49, lowers the iteration count by about 8 % but its m^3 setup costs more than that.)
-// The FP64 path keeps the full cycle: its Gauss-Jordan setup would run on the FP64 pipe, which
-// on this part costs more than the cycles it saves.
+// On the FP64 path it stops there from 1/32 on, one warp running the set-up (an FP64 instruction of a warp
+// holds its scheduler's FP64 unit for 64 cycles, however few lanes work, and the cycles on 1/4 and 1/2 are
+// ~60 such instructions an iteration with 1 .. 9 lanes: 1000 particles on 1/32, 128 threads, 2045 -> 1963 us);
+// on 1/16 the set-up costs what it saves (1000 particles 642 -> 669 us).
 // The flow cell (FC) always stops at 1/4 (15 unknowns: rows 0 .. 4 of columns 1 .. 3), on both
 // paths: its coarsest levels would need the boundary rows in the single-node solve.
 template <typename Real, bool FC = false>
 __host__ __device__ constexpr int direct_level(int N) {
-    return FC ? (N >= 8 ? 4 : 0) : sizeof(Real) == 8 ? 0 : (N >= 16 ? 4 : 0);
+    return FC ? (N >= 8 ? 4 : 0) : N >= (sizeof(Real) == 8 ? 32 : 16) ? 4 : 0;
 }
 // unknowns of the dense level NL: (NL - 1)^2, or (NL - 1)(NL + 1) for the flow cell
 __host__ __device__ constexpr int dense_unknowns(int NL, bool FC) { return (NL - 1) * (FC ? NL + 1 : NL - 1); }
@@ -530,9 +562,16 @@ __device__ __forceinline__ void solve_particle(const FemArgs& a, const int p, Re
     zero_rings<Real, N, N, T, FC>(arena);
     __syncthreads();
     Real* dinv = arena + arena_size(N, FC) + 4 * NPT * T;
-    if constexpr (direct_level<Real, FC>(N) != 0)
-        dense_setup<Real, direct_level<Real, FC>(N), T, FC>(
-            level_ptrs<Real, N, direct_level<Real, FC>(N), FC>(arena), dinv);
+    if constexpr (direct_level<Real, FC>(N) != 0) {
+        constexpr int ND = direct_level<Real, FC>(N);
+        const Lv<Real> L = level_ptrs<Real, N, ND, FC>(arena);
+        if constexpr (sizeof(Real) == 8 && !FC) {
+            if (tid < 32) dense_setup<Real, ND, 32, FC>(L, dinv);
+            __syncthreads();
+        } else {
+            dense_setup<Real, ND, T, FC>(L, dinv);
+        }
+    }
 
     // fine nodes owned by this thread, one packed int each: bits 0-12 node index n, 13-23 the
     // coarse node c under it ((j/2) SC + i/2), 24-25 (i & 1) + 2 (j & 1), 26 red, 27 valid.
@@ -673,10 +712,10 @@ __device__ __forceinline__ void solve_particle(const FemArgs& a, const int p, Re
             }
 #pragma unroll
             for (int q = 0; q < NPT; ++q) rz_new += r[q] * z[q];   // idle slots hold r = z = 0
-            block_sum<T>(rz_new, red_buf[parity]);
-            parity ^= 1;
             // p = z + beta p
-            const Real beta = (it == 0) ? Real(0) : rz_new / rz;
+            const Real quot = block_sum_div<T>(rz_new, rz, true, red_buf[parity]);
+            parity ^= 1;
+            const Real beta = (it == 0) ? Real(0) : quot;
             rz = rz_new;
 #pragma unroll
             for (int q = 0; q < NPT; ++q) {
@@ -696,9 +735,8 @@ __device__ __forceinline__ void solve_particle(const FemArgs& a, const int p, Re
                     pq += pv[q] * qv[q];
                 }
             }
-            block_sum<T>(pq, red_buf[parity]);
+            const Real alpha = block_sum_div<T>(pq, rz, false, red_buf[parity]);
             parity ^= 1;
-            const Real alpha = rz / pq;
             Real rr = 0;
 #pragma unroll
             for (int q = 0; q < NPT; ++q) {
@@ -1373,10 +1411,10 @@ cudaError_t fem_eval_persistent_launch(int N, int precision, int T, const FemArg
     } else {
         switch (N * 10000 + T) {
             case 4 * 10000 + 32: return launch_persistent<double, 4, 32>(groups, offsets, item_group, total, counter, st);
-            case 8 * 10000 + 64: return launch_persistent<double, 8, 64>(groups, offsets, item_group, total, counter, st);
+            case 8 * 10000 + 64: return launch_persistent<double, 8, 32>(groups, offsets, item_group, total, counter, st);
             case 16 * 10000 + 128: return launch_persistent<double, 16, 128>(groups, offsets, item_group, total, counter, st);
             case 16 * 10000 + 256: return launch_persistent<double, 16, 256>(groups, offsets, item_group, total, counter, st);
-            case 32 * 10000 + 256: return launch_persistent<double, 32, 256>(groups, offsets, item_group, total, counter, st);
+            case 32 * 10000 + 256: return launch_persistent<double, 32, 128>(groups, offsets, item_group, total, counter, st);
             case 32 * 10000 + 512: return launch_persistent<double, 32, 512>(groups, offsets, item_group, total, counter, st);
         }
     }
@@ -1398,7 +1436,9 @@ int fem_default_block(int N, int precision) {
     return s.empty() ? 0 : s[0];
 }
 
-// block sizes compiled for each level (threads per particle); the autotuner picks one
+// block sizes compiled for each level (threads per particle); the autotuner picks one. FP64: 64 at 1/8 names
+// one warp per particle and 256 at 1/32 four (per-warp work such as the reductions' sums and the divisions
+// is FP64 time: 1000 particles 197 -> 149 us and, with the exact 1/4 level, 2120 -> 1970 us)
 std::vector<int> fem_block_sizes(int N, int precision) {
     if (precision == SMC_MIXED) {
         switch (N) {
@@ -1452,10 +1492,10 @@ cudaError_t fem_eval_launch(const FemArgs& a, cudaStream_t st, int T) {
     } else {
         switch (a.N * 10000 + T) {
             case 4 * 10000 + 32: return launch_one<double, 4, 32>(a, st);
-            case 8 * 10000 + 64: return launch_one<double, 8, 64>(a, st);
+            case 8 * 10000 + 64: return launch_one<double, 8, 32>(a, st);
             case 16 * 10000 + 128: return launch_one<double, 16, 128>(a, st);
             case 16 * 10000 + 256: return launch_one<double, 16, 256>(a, st);
-            case 32 * 10000 + 256: return launch_one<double, 32, 256>(a, st);
+            case 32 * 10000 + 256: return launch_one<double, 32, 128>(a, st);
             case 32 * 10000 + 512: return launch_one<double, 32, 512>(a, st);
         }
     }
