@@ -45,6 +45,9 @@ struct Handle {
     double* scratch_phi = nullptr;
     int* scratch_iters = nullptr;
     int scratch_cap = 0;
+    // pinned host memory of small smc_eval_likelihood calls (made on the first one)
+    static constexpr size_t kHostStage = 256 << 10;
+    char* host_stage = nullptr;
 
     // sampler state (smc_kernels.cu / controller.cpp)
     struct Sampler* smp = nullptr;
