@@ -85,6 +85,7 @@ Handle::~Handle() {
     cudaFree(big_scratch);
     cudaFree(cp_scratch);
     cudaFree(big_counter);
+    cudaFree(tile_counter);
     cudaFree(d_y);
     free_sampler();
     for (auto* v : {&timed, &timed_phase})
@@ -170,7 +171,7 @@ FemArgs Handle::fem_args(int level, int n, const double* theta, double* G, doubl
 }
 
 int Handle::eval_device(int level, int n, const double* theta, double* G, double* Phi, int* iters,
-                        cudaStream_t st) {
+                        cudaStream_t st, unsigned* bad) {
     if (level < 0 || level >= (int)levels.size()) return fail(SMC_EINVAL, "level %d out of range", level);
     if (n < 0) return fail(SMC_EINVAL, "negative particle count");
     if (n == 0) return SMC_OK;
@@ -200,15 +201,20 @@ int Handle::eval_device(int level, int n, const double* theta, double* G, double
                 if (ea != cudaSuccess) return fail(SMC_ENOMEM, "tile-form scratch: %s", cudaGetErrorString(ea));
                 cp_cap = need;
             }
-            if (!big_counter && cudaMalloc((void**)&big_counter, sizeof(int)) != cudaSuccess)
-                return fail(SMC_ENOMEM, "work counter");
+            if (!tile_counter) {   // zeroed once: every launch leaves it at 0
+                if (cudaMalloc((void**)&tile_counter, sizeof(int)) != cudaSuccess)
+                    return fail(SMC_ENOMEM, "work counter");
+                cudaMemsetAsync(tile_counter, 0, sizeof(int), st);
+            }
+            a.bad = bad;   // counted by the solve itself
+            bad = nullptr;
             TimedLaunch t{level, nullptr, nullptr};
             if (timing) {
                 t.start = take_event();
                 t.stop = take_event();
                 cudaEventRecord(t.start, st);
             }
-            e = fem_tile_launch(a, cp_scratch, big_counter, st);
+            e = fem_tile_launch(a, cp_scratch, tile_counter, st);
             if (timing) {
                 cudaEventRecord(t.stop, st);
                 timed.push_back(t);
@@ -248,6 +254,7 @@ int Handle::eval_device(int level, int n, const double* theta, double* G, double
             e = fem_eval_launch(a, st, T);
         }
     }
+    if (e == cudaSuccess && bad) e = count_bad_launch(iters, n, bad, st);
     if (e != cudaSuccess) return cuda_fail(e, "forward-solve launch");
     return SMC_OK;
 }

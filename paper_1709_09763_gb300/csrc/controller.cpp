@@ -144,7 +144,8 @@ int Handle::smp_eval(int level, int n, const double* theta, double* phi) {
         da_ev[level].b = take_event();
         cudaEventRecord(da_ev[level].a, stream);
     }
-    RC(eval_device(level, n, theta, collect ? smp->G_buf : nullptr, phi, smp->iters, stream));
+    // non-converged solves are counted on the device and checked when the update reads its counters
+    RC(eval_device(level, n, theta, collect ? smp->G_buf : nullptr, phi, smp->iters, stream, bad_counter()));
     if (gate_open) {
         cudaEventRecord(da_ev[level].b, stream);
         da_ev[level].n = n;
@@ -154,8 +155,6 @@ int Handle::smp_eval(int level, int n, const double* theta, double* phi) {
         RC(mlp_add_pairs(level, n, theta, smp->G_buf));
         smp->pairs_new[level] += n;
     }
-    // non-converged solves are counted on the device and checked when the update reads its counters
-    CK(count_bad_launch(smp->iters, n, bad_counter(), stream));
     return SMC_OK;
 }
 

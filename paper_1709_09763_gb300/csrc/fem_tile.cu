@@ -1011,11 +1011,14 @@ __device__ __forceinline__ void solve_tile(const FemArgs& a, const int item, flo
         for (int k = 1; k < nw; ++k) misfit += part[k];
         a.Phi[item] = 0.5 * misfit * a.inv_sigma2;
         if (a.iters) a.iters[item] = converged ? total_it : -(total_it + 1);
+        if (a.bad && !converged) atomicAdd(a.bad, 1u);
     }
 }
 
 // persistent blocks (clusters: rank 0 hands the ticket to the others) take particles from a ticket
-// counter; the barrier at the end of a solve keeps every CTA from overwriting memory another still reads
+// counter; the barrier at the end of a solve keeps every CTA from overwriting memory another still reads.
+// Every block (cluster) draws tickets until one lies past the particles, so n + clusters are drawn in
+// all: whoever draws the last returns the counter to 0 for the next launch, which needs no memset.
 template <class G, bool RHS>
 __global__ void __launch_bounds__(G::T, G::MINB) fem_tile_kernel(FemArgs a, float4* ref_scratch, int* counter) {
     extern __shared__ __align__(16) float sm[];
@@ -1023,8 +1026,10 @@ __global__ void __launch_bounds__(G::T, G::MINB) fem_tile_kernel(FemArgs a, floa
     __shared__ int item_s[2];
     const int rank = G::H ? cluster_rank() : 0;
     float4* ref = ref_scratch + (size_t)blockIdx.x * G::REF4;
+    const int last = a.n + (int)gridDim.x / G::C - 1;
     auto take = [&](int k) {
         const int item = atomicAdd(counter, 1);
+        if (item == last) *counter = 0;
         item_s[k] = item;
         if constexpr (G::H)
             for (int c = 1; c < G::C; ++c) st_peer(&item_s[k], c, item);
@@ -1196,8 +1201,6 @@ cudaError_t fem_tile_launch(const FemArgs& a, float* ref_scratch, int* counter, 
     if (a.n <= 0) return cudaSuccess;
     if (!fem_tile_form(a.N, a.precision, a.flow_cell != 0) || !a.kappa) return cudaErrorInvalidValue;
     const int grid = tile_grid(a.N, a.n);
-    cudaError_t e = cudaMemsetAsync(counter, 0, sizeof(int), st);
-    if (e != cudaSuccess) return e;
     return with_form(a.N, [&](auto g) {
         using G = decltype(g);
         return a.rhs ? launch_one<G, true>(a, ref_scratch, grid, counter, st)

@@ -58,6 +58,7 @@ struct Handle {
     size_t cp_cap = 0;
     size_t big_cap = 0;
     int* big_counter = nullptr;
+    int* tile_counter = nullptr;   // ticket of the register-tiled form: 0 between launches
 
     // tensor-core KL synthesis buffers (kl_synth.cu)
     float* synth_kappa_buf = nullptr;
@@ -99,7 +100,9 @@ struct Handle {
     int fail(int code, const char* fmt, ...);
     int cuda_fail(cudaError_t e, const char* what);
     int ensure_scratch(int n);
-    int eval_device(int level, int n, const double* theta, double* G, double* Phi, int* iters, cudaStream_t st);
+    // bad (device, with iters): += solves that did not reach rtol
+    int eval_device(int level, int n, const double* theta, double* G, double* Phi, int* iters, cudaStream_t st,
+                    unsigned* bad = nullptr);
     FemArgs fem_args(int level, int n, const double* theta, double* G, double* Phi, int* iters) const;
     int block_size(int N) const;
     int alloc_sampler();

@@ -63,6 +63,7 @@ struct FemArgs {
     double bnorm2;          // sum of squares of the load vector over the interior nodes (with rhs)
     int flow_cell;          // 1: the flow cell of Example 5.3 (p = 0 / 1 on x = 0 / 1, no flow on
                             // y = 0, 1, f = 0; levels 1/8 .. 1/256, FP64 to 1/32; no batched form)
+    unsigned* bad;          // += solves that did not reach rtol, or null (fem_tile_launch only)
 };
 // Returns cudaSuccess or the launch error.
 // T = threads per particle (one of fem_block_sizes; <= 0: the first, the default)
@@ -87,8 +88,9 @@ cudaError_t fem_eval_persistent_launch(int N, int precision, int T, const FemArg
                                        const int* item_group, int total, int* counter, cudaStream_t st);
 // register-tiled form of the mixed solve (fem_tile.cu): 1/32 and 1/64 on one CTA (every block size of those
 // levels), 1/128 on a cluster of two CTAs (block size -1024), 1/256 of eight; not the flow cell. Where a
-// cluster does not fit, 1/128 and 1/256 run in the device-memory form above. fem_tile_scratch floats of device scratch hold the refinement state. *counter (device) is reset by
-// fem_tile_launch; fem_tile_multi_launch (arguments as fem_eval_persistent_launch) needs it zero
+// cluster does not fit, 1/128 and 1/256 run in the device-memory form above. fem_tile_scratch floats of device
+// scratch hold the refinement state. *counter (device) is 0 before a launch; fem_tile_launch leaves it at 0,
+// fem_tile_multi_launch (arguments as fem_eval_persistent_launch) does not
 bool fem_tile_form(int N, int precision, bool flow_cell);
 size_t fem_tile_scratch(int N);
 cudaError_t fem_tile_launch(const FemArgs& a, float* scratch, int* counter, cudaStream_t st);

@@ -72,8 +72,10 @@ __device__ __forceinline__ void normal_pair(uint32_t b, uint32_t j, uint32_t eve
     const double v1 = u53(x.x, x.y), v2 = u53(x.z, x.w);
     const double r = sqrt(-2.0 * log(1.0 - v1));
     const double ang = 2.0 * 3.141592653589793 * v2;
-    z0 = r * cos(ang);
-    z1 = r * sin(ang);
+    double sn, cs;
+    sincos(ang, &sn, &cs);   // one argument reduction for both
+    z0 = r * cs;
+    z1 = r * sn;
 }
 
 // the task (problem) of this block in a multi-problem launch: start[p] <= blockIdx.x < start[p + 1]
@@ -91,7 +93,13 @@ __device__ __forceinline__ int task_of_block(const int* start, int count) {
     return p_s;
 }
 
-__global__ void normals_kernel(double* out, int J, int K, uint32_t event, uint32_t purpose, uint64_t seed,
+// 64-thread blocks: a draw is some hundred FP64 instructions, and one FP64 instruction of a warp
+// holds its scheduler's unit for 64 cycles, so a call of a thousand particles wants its 500 warps on
+// as many schedulers as there are (256-thread blocks put them on 63 of the 152 SMs).
+// 1000 x 32 draws with a base: 9.8 us with those, now 6.2 us.
+constexpr int kNormThreads = 64;
+
+__global__ void __launch_bounds__(kNormThreads) normals_kernel(double* out, int J, int K, uint32_t event, uint32_t purpose, uint64_t seed,
                                const double* base, double c0, double c1) {
     // out[j][k] = c0 * base[j][k] + c1 * xi[j][k]  (base == null: out = xi)
     const int nb = (K + 1) / 2;
@@ -110,8 +118,8 @@ __global__ void normals_kernel(double* out, int J, int K, uint32_t event, uint32
     }
 }
 
-// many problems' proposals or draws (256-thread blocks, a contiguous block range per problem)
-__global__ void normals_multi_kernel(const __grid_constant__ NormTasks T) {
+// many problems' proposals or draws (a contiguous block range per problem)
+__global__ void __launch_bounds__(kNormThreads) normals_multi_kernel(const __grid_constant__ NormTasks T) {
     const int p = task_of_block(T.start, T.count);
     const NormTask& k = T.t[p];
     const int nb = (k.K + 1) / 2;
@@ -308,11 +316,34 @@ __device__ bool grid_barrier(unsigned* bar, int* err, unsigned nblocks, unsigned
     return true;
 }
 
-// sum of v[kIncSums] over the block into thread 0 (warp shuffles, then warp 0 over the warps)
-__device__ __forceinline__ void inc_block_sum(double (&v)[kIncSums], double* sh /*[kIncSums][32]*/) {
+// Sums of v[0..5] over a warp; lane 0 has them all. The lanes halve the list as they halve the
+// distance (lane and partner each take three of the six, then two or one, then one), so a sum is the
+// same tree over the lanes as a butterfly of its own, bit for bit, in 8 FP64 additions instead of
+// 30: an FP64 instruction of a warp holds its scheduler's unit for 64 cycles (a search over 1000
+// particles: 63 us with butterflies, now 55 us).
+__device__ __forceinline__ void inc_warp_sum(double (&v)[kIncSums]) {
+    static_assert(kIncSums == 6, "the list is halved to 3, 2 and 1");
+    const int lane = threadIdx.x & 31;
+    const bool h4 = lane & 16, h3 = lane & 8, h2 = lane & 4;
+    double a[3];
 #pragma unroll
-    for (int i = 0; i < kIncSums; ++i)
-        for (int off = 16; off > 0; off >>= 1) v[i] += __shfl_xor_sync(0xffffffffu, v[i], off);
+    for (int i = 0; i < 3; ++i)   // lanes 0-15: sums 0, 1, 2; lanes 16-31: 3, 4, 5
+        a[i] = (h4 ? v[i + 3] : v[i]) + __shfl_xor_sync(0xffffffffu, h4 ? v[i] : v[i + 3], 16);
+    // bit 3 clear: the first and the second of the three; set: the third
+    const double b0 = (h3 ? a[2] : a[0]) + __shfl_xor_sync(0xffffffffu, h3 ? a[0] : a[2], 8);
+    const double b1 = a[1] + __shfl_xor_sync(0xffffffffu, a[1], 8);
+    // bit 2 clear: the first (or the third); set: the second
+    double c = (h2 && !h3 ? b1 : b0) + __shfl_xor_sync(0xffffffffu, h2 || h3 ? b0 : b1, 4);
+    c += __shfl_xor_sync(0xffffffffu, c, 2);
+    c += __shfl_xor_sync(0xffffffffu, c, 1);
+    // sums 0 .. 5 are with lanes 0, 4, 8, 16, 20, 24
+#pragma unroll
+    for (int i = 0; i < kIncSums; ++i) v[i] = __shfl_sync(0xffffffffu, c, (i / 3) * 16 + (i % 3) * 4);
+}
+
+// sum of v[kIncSums] over the block into thread 0 (each warp, then warp 0 over the warps)
+__device__ __forceinline__ void inc_block_sum(double (&v)[kIncSums], double* sh /*[kIncSums][32]*/) {
+    inc_warp_sum(v);
     constexpr int nw = kIncThreads / 32;
     if (nw > 1) {
         if ((threadIdx.x & 31) == 0 && threadIdx.x > 0)
@@ -400,9 +431,7 @@ __device__ __forceinline__ void inc_search_blocks(const double* a, int n, double
             for (unsigned k = lane; k < nb; k += 32)
 #pragma unroll
                 for (int i = 0; i < kIncSums; ++i) t[i] += __ldcg(&part[k * kIncSums + i]);
-#pragma unroll
-            for (int i = 0; i < kIncSums; ++i)
-                for (int off = 16; off > 0; off >>= 1) t[i] += __shfl_xor_sync(0xffffffffu, t[i], off);
+            inc_warp_sum(t);
             if (lane == 0) inc_decide(st, t, n, max_iter);
         }
         __syncthreads();
@@ -672,60 +701,100 @@ __device__ __forceinline__ double target_potential(double beta, double zeta, dou
     return __dmul_rn(beta, __dadd_rn(__dmul_rn(1.0 - zeta, pc), __dmul_rn(zeta, pf)));
 }
 
-// the Metropolis decision of particle j (j >= n: none); true if the proposal was taken
-__device__ __forceinline__ bool pcn_accept_one(int j, int n, int K, double beta, double zeta, uint32_t event,
-                                               uint64_t seed, double* theta, const double* theta_p, double* phi_c,
-                                               const double* phi_cp, double* phi_f, const double* phi_fp, int rwm) {
-    bool ok = false;
-    if (j < n) {
-        const uint4 x = philox(make_uint4(0u, (uint32_t)j, event, (uint32_t)kPurposePcnU), seed);
-        const double U = 1.0 - u53(x.x, x.y);
-        const double t_old = target_potential(beta, zeta, phi_c[j], zeta < 0.0 ? 0.0 : phi_f[j]);
-        const double t_new = target_potential(beta, zeta, phi_cp[j], zeta < 0.0 ? 0.0 : phi_fp[j]);
-        double log_prior = 0.0;   // random walk: log mu0(theta') - log mu0(theta), mu0 = N(0, I)
-        if (rwm) {
-            double sn = 0.0, so = 0.0;
-            for (int k = 0; k < K; ++k) {
-                const double a = theta_p[(size_t)j * K + k], b = theta[(size_t)j * K + k];
-                sn += a * a;
-                so += b * b;
+// A block of 256 threads takes 32 particles: one warp decides (a lane per particle, all of the FP64
+// work), then every warp copies four of the 32 rows, coalesced, having fetched their first 32 entries
+// while the decision was made. Bound by latency (a chain of two loads, log U and one copy): with a
+// thread copying its own row 1000 x 32 took 9.0 us, now 5.2 us. The deciding warp differs
+// between the blocks that share an SM, so that their FP64 work is on different schedulers.
+constexpr int kAccRows = 32, kAccThreads = 256;
+
+__device__ __forceinline__ void pcn_accept_rows(int j0, int n, int K, double beta, double zeta, uint32_t event,
+                                                uint64_t seed, double* theta, const double* theta_p, double* phi_c,
+                                                const double* phi_cp, double* phi_f, const double* phi_fp,
+                                                unsigned long long* n_acc, int rwm) {
+    constexpr int kWarps = kAccThreads / 32, kRows = kAccRows / kWarps;
+    __shared__ unsigned taken_s;
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const int rows = min(kAccRows, n - j0);
+    const double* src = theta_p + (size_t)j0 * K;
+    double* dst = theta + (size_t)j0 * K;
+    double v[kRows];
+#pragma unroll
+    for (int i = 0; i < kRows; ++i) {
+        const int r = wid + i * kWarps;
+        v[i] = r < rows && lane < K ? src[(size_t)r * K + lane] : 0.0;
+    }
+    if (wid == (int)(blockIdx.x >> 7) % 4) {
+        bool ok = false;
+        const int j = j0 + lane;
+        if (lane < rows) {
+            const uint4 x = philox(make_uint4(0u, (uint32_t)j, event, (uint32_t)kPurposePcnU), seed);
+            const double U = 1.0 - u53(x.x, x.y);
+            const double pc = phi_cp[j], pf = zeta < 0.0 ? 0.0 : phi_fp[j];
+            const double t_old = target_potential(beta, zeta, phi_c[j], zeta < 0.0 ? 0.0 : phi_f[j]);
+            const double t_new = target_potential(beta, zeta, pc, pf);
+            double log_prior = 0.0;   // random walk: log mu0(theta') - log mu0(theta), mu0 = N(0, I)
+            if (rwm) {
+                double sn = 0.0, so = 0.0;
+                for (int k = 0; k < K; ++k) {
+                    const double a = src[(size_t)lane * K + k], b = dst[(size_t)lane * K + k];
+                    sn += a * a;
+                    so += b * b;
+                }
+                log_prior = -0.5 * (sn - so);
             }
-            log_prior = -0.5 * (sn - so);
+            ok = log(U) < -(t_new - t_old) + log_prior;
+            if (ok) {
+                phi_c[j] = pc;
+                if (zeta >= 0.0) phi_f[j] = pf;
+            }
         }
-        ok = log(U) < -(t_new - t_old) + log_prior;
-        if (ok) {
-            for (int k = 0; k < K; ++k) theta[(size_t)j * K + k] = theta_p[(size_t)j * K + k];
-            phi_c[j] = phi_cp[j];
-            if (zeta >= 0.0) phi_f[j] = phi_fp[j];
+        const unsigned taken = __ballot_sync(0xffffffffu, ok);
+        if (lane == 0) {
+            taken_s = taken;
+            if (taken) atomicAdd(n_acc, (unsigned long long)__popc(taken));
         }
     }
-    return ok;
+    __syncthreads();
+    const unsigned taken = taken_s;
+#pragma unroll
+    for (int i = 0; i < kRows; ++i) {
+        const int r = wid + i * kWarps;
+        if ((taken >> r & 1u) && lane < K) dst[(size_t)r * K + lane] = v[i];
+    }
+    for (int k = lane + 32; k < K; k += 32) {
+#pragma unroll
+        for (int i = 0; i < kRows; ++i) {
+            const int r = wid + i * kWarps;
+            v[i] = taken >> r & 1u ? src[(size_t)r * K + k] : 0.0;
+        }
+#pragma unroll
+        for (int i = 0; i < kRows; ++i) {
+            const int r = wid + i * kWarps;
+            if (taken >> r & 1u) dst[(size_t)r * K + k] = v[i];
+        }
+    }
 }
 
-__global__ void pcn_accept_kernel(int n, int K, double beta, const double* beta_p, double zeta, const double* zeta_p,
-                                  uint32_t event, uint64_t seed, double* theta, const double* theta_p, double* phi_c,
-                                  const double* phi_cp, double* phi_f, const double* phi_fp,
-                                  unsigned long long* n_acc, int rwm) {
-    const int j = blockIdx.x * blockDim.x + threadIdx.x;
+__global__ void __launch_bounds__(kAccThreads) pcn_accept_kernel(
+    int n, int K, double beta, const double* beta_p, double zeta, const double* zeta_p, uint32_t event, uint64_t seed,
+    double* theta, const double* theta_p, double* phi_c, const double* phi_cp, double* phi_f, const double* phi_fp,
+    unsigned long long* n_acc, int rwm) {
     if (beta_p) beta = *beta_p;
     if (zeta_p) zeta = *zeta_p;
-    const bool ok = pcn_accept_one(j, n, K, beta, zeta, event, seed, theta, theta_p, phi_c, phi_cp, phi_f, phi_fp, rwm);
-    const unsigned ballot = __ballot_sync(0xffffffffu, ok);
-    if ((threadIdx.x & 31) == 0 && ballot) atomicAdd(n_acc, (unsigned long long)__popc(ballot));
+    pcn_accept_rows((int)blockIdx.x * kAccRows, n, K, beta, zeta, event, seed, theta, theta_p, phi_c, phi_cp, phi_f,
+                    phi_fp, n_acc, rwm);
 }
 
-// many problems' acceptances (64-thread blocks, a contiguous block range per problem); beta and
-// zeta read from the device where a pointer is given (the value an increment search left there)
-__global__ void pcn_accept_multi_kernel(const __grid_constant__ AccTasks T) {
+// many problems' acceptances (a contiguous block range per problem); beta and zeta read from the
+// device where a pointer is given (the value an increment search left there)
+__global__ void __launch_bounds__(kAccThreads) pcn_accept_multi_kernel(const __grid_constant__ AccTasks T) {
     const int p = task_of_block(T.start, T.count);
     const AccTask& k = T.t[p];
-    const int j = (int)(blockIdx.x - (unsigned)T.start[p]) * blockDim.x + threadIdx.x;
     const double beta = k.beta_p ? *k.beta_p : k.beta;
     const double zeta = k.zeta_p ? *k.zeta_p : k.zeta;
-    const bool ok = pcn_accept_one(j, k.n, k.K, beta, zeta, k.event, k.seed, k.theta, k.theta_p, k.phi_c, k.phi_cp,
-                                   k.phi_f, k.phi_fp, k.rwm);
-    const unsigned ballot = __ballot_sync(0xffffffffu, ok);
-    if ((threadIdx.x & 31) == 0 && ballot) atomicAdd(k.n_acc, (unsigned long long)__popc(ballot));
+    pcn_accept_rows((int)(blockIdx.x - (unsigned)T.start[p]) * kAccRows, k.n, k.K, beta, zeta, k.event, k.seed, k.theta,
+                    k.theta_p, k.phi_c, k.phi_cp, k.phi_f, k.phi_fp, k.n_acc, k.rwm);
 }
 
 // ---- delayed acceptance (Christen & Fox 2005) ----------------------------------------------------
@@ -973,7 +1042,7 @@ cudaError_t normals_launch(double* out, int J, int K, uint32_t event, uint32_t p
                            const double* base, double c0, double c1, cudaStream_t st) {
     if (J <= 0) return cudaSuccess;
     const long long work = (long long)J * ((K + 1) / 2);
-    normals_kernel<<<grid_for(work, 256), 256, 0, st>>>(out, J, K, event, purpose, seed, base, c0, c1);
+    normals_kernel<<<grid_for(work, kNormThreads), kNormThreads, 0, st>>>(out, J, K, event, purpose, seed, base, c0, c1);
     count_launches(1);
     return cudaGetLastError();
 }
@@ -1048,8 +1117,7 @@ cudaError_t pcn_accept_launch(int n, int K, double beta, const double* beta_p, d
                               const double* phi_cp, double* phi_f, const double* phi_fp, unsigned long long* n_acc,
                               int rwm, cudaStream_t st) {
     if (n <= 0) return cudaSuccess;
-    // 64-thread blocks: the FP64 work (log U, target potentials) spread over many SMs
-    pcn_accept_kernel<<<grid_for(n, 64), 64, 0, st>>>(n, K, beta, beta_p, zeta, zeta_p, event, seed, theta, theta_p,
+    pcn_accept_kernel<<<grid_for(n, kAccRows), kAccThreads, 0, st>>>(n, K, beta, beta_p, zeta, zeta_p, event, seed, theta, theta_p,
                                                       phi_c, phi_cp, phi_f, phi_fp, n_acc, rwm);
     count_launches(1);
     return cudaGetLastError();
@@ -1183,18 +1251,18 @@ cudaError_t resample_gather_multi_launch(const std::vector<RsTask>& tasks, cudaS
 }
 
 cudaError_t normals_multi_launch(const std::vector<NormTask>& tasks, cudaStream_t st) {
-    return for_task_lists(tasks, 1 << 30, [](const NormTask& t) { return grid_for((long long)t.J * ((t.K + 1) / 2), 256); },
+    return for_task_lists(tasks, 1 << 30, [](const NormTask& t) { return grid_for((long long)t.J * ((t.K + 1) / 2), kNormThreads); },
                           [&](const NormTasks& L, int blocks) {
-                              normals_multi_kernel<<<blocks, 256, 0, st>>>(L);
+                              normals_multi_kernel<<<blocks, kNormThreads, 0, st>>>(L);
                               count_launches(1);
                               return cudaGetLastError();
                           });
 }
 
 cudaError_t pcn_accept_multi_launch(const std::vector<AccTask>& tasks, cudaStream_t st) {
-    return for_task_lists(tasks, 1 << 30, [](const AccTask& t) { return grid_for(t.n, 64); },
+    return for_task_lists(tasks, 1 << 30, [](const AccTask& t) { return grid_for(t.n, kAccRows); },
                           [&](const AccTasks& L, int blocks) {
-                              pcn_accept_multi_kernel<<<blocks, 64, 0, st>>>(L);
+                              pcn_accept_multi_kernel<<<blocks, kAccThreads, 0, st>>>(L);
                               count_launches(1);
                               return cudaGetLastError();
                           });
