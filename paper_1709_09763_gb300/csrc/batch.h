@@ -13,6 +13,27 @@
 namespace mls2mc {
 
 struct BatchSampler;
+
+// Streams beside a batch's own: during a capture they make parallel branches of the graph.
+struct Forks {
+    static constexpr int kMax = 16;
+    cudaStream_t s[kMax] = {};
+    cudaEvent_t start = nullptr, end[kMax] = {};
+    bool ready();   // makes them on first use; false: no streams to be had
+    // s[0 .. n - 1] begin where st is; st goes on when they are done
+    cudaError_t fork(int n, cudaStream_t st);
+    cudaError_t join(int n, cudaStream_t st);
+    ~Forks();
+};
+
+// the syntheses of many problems (each of its own handle): one split launch, then a contraction per problem, on
+// parallel branches where forks are given. Returns SMC_OK or the failing problem's code (*err: its message).
+struct SynthReq {
+    Handle* h;
+    int level, n;
+    const double* theta;
+};
+int synth_many(const std::vector<SynthReq>& reqs, Forks* forks, cudaStream_t st, std::string* err);
 void batch_sampler_free(BatchSampler* s);
 
 struct Batch {
@@ -32,6 +53,7 @@ struct Batch {
     cudaGraph_t graph = nullptr;
     cudaGraphExec_t exec = nullptr;
     long long graph_kernels = 0;
+    Forks forks;
     std::string last_error;
     BatchSampler* smp = nullptr;   // state of the batched sampler, made on its first step
     bool owns_handles = false;     // made by smc_init_batch: the handles are destroyed with the batch

@@ -145,6 +145,13 @@ int multi_eval(Batch* b, const std::vector<EvalReq>& reqs, cudaStream_t st) {
             int N, precision, T, first, count, total, item_base;
         };
         std::vector<G> groups;
+        std::vector<SynthReq> synth;
+        for (const size_t i : idx) {
+            Handle* h = b->h[reqs[i].p];
+            if (h->precision == SMC_MIXED) synth.push_back({h, reqs[i].level, reqs[i].n, reqs[i].theta});
+        }
+        const int rc = synth_many(synth, nullptr, st, &b->last_error);
+        if (rc != SMC_OK) return rc;
         int items = 0;
         for (size_t r = 0; r < idx.size(); ++r) {
             const EvalReq& q = reqs[idx[r]];
@@ -155,11 +162,7 @@ int multi_eval(Batch* b, const std::vector<EvalReq>& reqs, cudaStream_t st) {
             }
             G& g = groups.back();
             FemArgs a = h->fem_args(q.level, q.n, q.theta, nullptr, q.phi, h->smp->iters);
-            if (h->precision == SMC_MIXED) {
-                const int rc = h->synth_kappa(q.level, q.n, q.theta, st);
-                if (rc != SMC_OK) return bfail(b, rc, h->last_error);
-                a.kappa = h->synth_kappa_buf;
-            }
+            if (h->precision == SMC_MIXED) a.kappa = h->synth_kappa_buf;
             U.args[r] = a;
             U.offsets[r] = g.total;
             U.rel[r] = g.count;

@@ -67,7 +67,8 @@ struct Handle {
     float* synth_part_buf = nullptr;   // K > 256: FP32 partial fields of the term groups [groups][n][E]
     size_t synth_part_cap = 0;
     int* synth_err = nullptr;
-    int synth_kappa(int level, int n, const double* theta, cudaStream_t st);
+    // split: false where theta_split_multi_launch has split theta already (one contraction only)
+    int synth_kappa(int level, int n, const double* theta, cudaStream_t st, bool split = true);
     int synth_reserve(int level, int n);
 
     // opt-in CUDA-event timing of forward-solve launches, per level

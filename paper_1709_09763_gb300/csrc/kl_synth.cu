@@ -30,6 +30,7 @@
 #include <vector>
 
 #include "handle.h"
+#include "smc_device.h"
 #include "umma_gemm.h"
 
 namespace mls2mc {
@@ -44,14 +45,10 @@ namespace {
 // 4000 x 32 with a thread per output and its 64-bit division, now 3.5 us.
 constexpr int kSplitThreads = 128;
 
+// the split of one particle's terms th into its row, by threads x = 0 .. kx - 1
 template <int V>
-__global__ void __launch_bounds__(kSplitThreads)
-    theta_split_kernel(const double* theta, int n, int K, int k0, int Kg, int Kp, __nv_bfloat16* out) {
-    const long long j = (long long)blockIdx.x * blockDim.y + threadIdx.y;
-    if (j >= n) return;
-    const double* th = theta + (size_t)j * K + k0;
-    __nv_bfloat16* row = out + (size_t)j * Kp;
-    for (int k = (int)threadIdx.x * V; k < Kg; k += (int)blockDim.x * V) {
+__device__ __forceinline__ void split_row(const double* th, int Kg, int Kp, int x0, int kx, __nv_bfloat16* row) {
+    for (int k = x0 * V; k < Kg; k += kx * V) {
         __nv_bfloat16 p1[V], p2[V], p3[V];
 #pragma unroll
         for (int i = 0; i < V; ++i) {
@@ -75,7 +72,29 @@ __global__ void __launch_bounds__(kSplitThreads)
                 *o = sel[b][0];
         }
     }
-    for (int c = 6 * Kg + (int)threadIdx.x; c < Kp; c += (int)blockDim.x) row[c] = __float2bfloat16_rn(0.0f);
+    for (int c = 6 * Kg + x0; c < Kp; c += kx) row[c] = __float2bfloat16_rn(0.0f);
+}
+
+template <int V>
+__global__ void __launch_bounds__(kSplitThreads)
+    theta_split_kernel(const double* theta, int n, int K, int k0, int Kg, int Kp, __nv_bfloat16* out) {
+    const long long j = (long long)blockIdx.x * blockDim.y + threadIdx.y;
+    if (j < n)
+        split_row<V>(theta + (size_t)j * K + k0, Kg, Kp, (int)threadIdx.x, (int)blockDim.x, out + (size_t)j * Kp);
+}
+
+// many problems' splits: blockIdx.y is the problem, the blocks in x stride over its particles
+__global__ void __launch_bounds__(kSplitThreads) theta_split_multi_kernel(const __grid_constant__ SplitTasks L) {
+    const SplitTask& t = L.t[blockIdx.y];
+    __nv_bfloat16* out = reinterpret_cast<__nv_bfloat16*>(t.out);
+    const bool pair = t.K % 2 == 0;
+    const int kx = min(pair ? t.K / 2 : t.K, kSplitThreads), ry = kSplitThreads / kx;
+    const int x = (int)threadIdx.x % kx, y = (int)threadIdx.x / kx;
+    if (y >= ry) return;
+    for (long long j = (long long)blockIdx.x * ry + y; j < t.n; j += (long long)gridDim.x * ry) {
+        if (pair) split_row<2>(t.theta + (size_t)j * t.K, t.K, t.Kp, x, kx, out + (size_t)j * t.Kp);
+        else split_row<1>(t.theta + (size_t)j * t.K, t.K, t.Kp, x, kx, out + (size_t)j * t.Kp);
+    }
 }
 
 void theta_split_launch(const double* theta, int n, int K, int k0, int Kg, int Kp, __nv_bfloat16* out, cudaStream_t st) {
@@ -194,12 +213,31 @@ int Handle::synth_reserve(int level, int n) {
     return SMC_OK;
 }
 
-int Handle::synth_kappa(int level, int n, const double* theta, cudaStream_t st) {
+cudaError_t theta_split_multi_launch(const std::vector<SplitTask>& tasks, cudaStream_t st) {
+    SplitTasks L;
+    for (size_t i0 = 0; i0 < tasks.size(); i0 += kMaxTasks) {
+        L.count = (int)std::min<size_t>(kMaxTasks, tasks.size() - i0);
+        int blocks = 1;
+        for (int i = 0; i < L.count; ++i) {
+            L.t[i] = tasks[i0 + i];
+            const int terms = L.t[i].K % 2 == 0 ? L.t[i].K / 2 : L.t[i].K, ry = kSplitThreads / std::min(terms, kSplitThreads);
+            blocks = std::max(blocks, std::min(64, (int)(((long long)L.t[i].n + ry - 1) / ry)));
+        }
+        theta_split_multi_kernel<<<dim3(blocks, L.count), kSplitThreads, 0, st>>>(L);
+        count_launches(1);
+        const cudaError_t e = cudaGetLastError();
+        if (e != cudaSuccess) return e;
+    }
+    return cudaSuccess;
+}
+
+int Handle::synth_kappa(int level, int n, const double* theta, cudaStream_t st, bool split) {
     const Level& L = levels[level];
     const int E = 2 * L.N * L.N, Kt = kl_split_total(K), G = kl_groups(K);
     RC_CHECK(synth_reserve(level, n));
     if (G == 1) {
-        theta_split_launch(theta, n, K, 0, K, Kt, reinterpret_cast<__nv_bfloat16*>(synth_theta_buf), st);
+        if (split)
+            theta_split_launch(theta, n, K, 0, K, Kt, reinterpret_cast<__nv_bfloat16*>(synth_theta_buf), st);
         GemmEpi epi;
         epi.kind = kEpiExp;
         epi.out_f32 = synth_kappa_buf;

@@ -137,6 +137,11 @@ struct CvTask {
     int n;
     double beta;
 };
+struct SplitTask {
+    const double* theta;
+    uint16_t* out;   // BF16 bits [n][Kp]
+    int n, K, Kp;
+};
 struct BadTask {
     const int* iters;
     unsigned* bad;
@@ -155,6 +160,7 @@ using AccTasks = TaskList<AccTask>;
 using LuTasks = TaskList<LuTask>;
 using CvTasks = TaskList<CvTask>;
 using BadTasks = TaskList<BadTask>;
+using SplitTasks = TaskList<SplitTask>;
 struct ZeroList {
     unsigned* ptr[2 * kMaxTasks];
     int words[2 * kMaxTasks];
@@ -168,6 +174,8 @@ cudaError_t normals_multi_launch(const std::vector<NormTask>& tasks, cudaStream_
 cudaError_t pcn_accept_multi_launch(const std::vector<AccTask>& tasks, cudaStream_t st);
 cudaError_t lu_increment_multi_launch(const std::vector<LuTask>& tasks, cudaStream_t st);
 cudaError_t cv_lu_multi_launch(const std::vector<CvTask>& tasks, cudaStream_t st);
+// theta splits of many problems' syntheses (kl_synth.cu; expansions of one contraction each)
+cudaError_t theta_split_multi_launch(const std::vector<SplitTask>& tasks, cudaStream_t st);
 cudaError_t count_bad_multi_launch(const std::vector<BadTask>& tasks, cudaStream_t st);
 // words (unsigned) to zero: (pointer, count) pairs
 cudaError_t zero_words_launch(const std::vector<std::pair<unsigned*, int>>& list, cudaStream_t st);
