@@ -54,7 +54,7 @@ struct Handle {
 
     // large levels: per-block hierarchy slices in global memory (fem_solve.cu)
     float* big_scratch = nullptr;
-    float* cp_scratch = nullptr;   // refinement state of the tile form's blocks and the two-CTA form's CTAs
+    float* cp_scratch = nullptr;   // refinement state of the register-tiled form's CTAs
     size_t cp_cap = 0;
     size_t big_cap = 0;
     int* big_counter = nullptr;
