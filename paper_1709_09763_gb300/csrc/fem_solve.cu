@@ -43,6 +43,7 @@
 #include <vector>
 
 #include "fem_device.h"
+#include "launch.h"
 #include "internal.h"
 
 namespace mls2mc {
@@ -1225,6 +1226,7 @@ __host__ __device__ constexpr int solve_min_blocks() {
 template <typename Real, int N, int T>
 __global__ void __launch_bounds__(T, (solve_min_blocks<Real, N, T>()))
 fem_eval_kernel(FemArgs a) {
+    grid_wait();
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ double red_buf[2][64];
     __shared__ Real theta_s[256];
@@ -1285,9 +1287,9 @@ cudaError_t launch_one(const FemArgs& a, cudaStream_t st) {
     auto kern = fem_eval_kernel<Real, N, T>;
     cudaError_t err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (err != cudaSuccess) return err;
-    kern<<<a.n, T, smem, st>>>(a);
+    err = launch_after(kern, dim3(a.n), dim3(T), smem, st, a);
     count_launches(1);
-    return cudaGetLastError();
+    return err != cudaSuccess ? err : cudaGetLastError();
 }
 
 template <typename Real, int N, int T>

@@ -44,6 +44,7 @@
 
 #include "fem_device.h"
 #include "internal.h"
+#include "launch.h"
 
 namespace mls2mc {
 
@@ -1026,6 +1027,7 @@ __global__ void __launch_bounds__(G::T, G::MINB) fem_tile_kernel(FemArgs a, floa
     __shared__ int item_s[2];
     const int rank = G::H ? cluster_rank() : 0;
     float4* ref = ref_scratch + (size_t)blockIdx.x * G::REF4;
+    grid_wait();
     const int last = a.n + (int)gridDim.x / G::C - 1;
     auto take = [&](int k) {
         const int item = atomicAdd(counter, 1);
@@ -1129,8 +1131,9 @@ cudaError_t launch_one(const FemArgs& a, float* ref_scratch, int grid, int* coun
     cudaError_t e = set_smem<G>(fem_tile_kernel<G, RHS>);
     if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg;
-    cudaLaunchAttribute attr;
-    config<G>(cfg, attr, grid, st);
+    cudaLaunchAttribute attr[2];
+    config<G>(cfg, attr[0], grid, st);
+    if (may_overlap(st)) overlap_attr(attr[cfg.numAttrs++]);
     e = cudaLaunchKernelEx(&cfg, fem_tile_kernel<G, RHS>, a, reinterpret_cast<float4*>(ref_scratch), counter);
     count_launches(1);
     return e != cudaSuccess ? e : cudaGetLastError();

@@ -30,6 +30,7 @@
 #include <vector>
 
 #include "handle.h"
+#include "launch.h"
 #include "smc_device.h"
 #include "umma_gemm.h"
 
@@ -78,6 +79,8 @@ __device__ __forceinline__ void split_row(const double* th, int Kg, int Kp, int 
 template <int V>
 __global__ void __launch_bounds__(kSplitThreads)
     theta_split_kernel(const double* theta, int n, int K, int k0, int Kg, int Kp, __nv_bfloat16* out) {
+    grid_wait();
+    grid_release();
     const long long j = (long long)blockIdx.x * blockDim.y + threadIdx.y;
     if (j < n)
         split_row<V>(theta + (size_t)j * K + k0, Kg, Kp, (int)threadIdx.x, (int)blockDim.x, out + (size_t)j * Kp);
@@ -102,10 +105,8 @@ void theta_split_launch(const double* theta, int n, int K, int k0, int Kg, int K
     const int kx = std::min(terms, kSplitThreads), ry = kSplitThreads / kx;
     const dim3 block(kx, ry);
     const unsigned grid = (unsigned)(((long long)n + ry - 1) / ry);
-    if (Kg % 2 == 0)
-        theta_split_kernel<2><<<grid, block, 0, st>>>(theta, n, K, k0, Kg, Kp, out);
-    else
-        theta_split_kernel<1><<<grid, block, 0, st>>>(theta, n, K, k0, Kg, Kp, out);
+    launch_after(Kg % 2 == 0 ? theta_split_kernel<2> : theta_split_kernel<1>, grid, block, 0, st, theta, n, K, k0, Kg, Kp,
+                 out);
     count_launches(1);
 }
 

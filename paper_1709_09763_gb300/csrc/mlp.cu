@@ -25,6 +25,7 @@
 #include "handle.h"
 #include "mlp.h"
 #include "smc_device.h"
+#include "launch.h"
 #include "umma_gemm.h"
 
 namespace mls2mc {
@@ -73,6 +74,8 @@ dim3 tile_grid(int B, int cols) {
 __global__ void __launch_bounds__(kTileThreads) input_kernel(const double* theta, int B, int K, int Kp, __nv_bfloat16* X,
                                                              __nv_bfloat16* Xt, int ldt) {
     __shared__ __align__(16) BatchTile tile;
+    grid_wait();
+    grid_release();
     const int b0 = blockIdx.x * kTileRows, c0 = blockIdx.y * kTileCols, cl = threadIdx.x % kTileCols, k = c0 + cl;
     double x[kTilePer];
 #pragma unroll
@@ -160,6 +163,8 @@ __global__ void __launch_bounds__(kTileThreads) loss_grad_kernel(const float* Z,
                                                                  double* partial) {
     __shared__ __align__(16) BatchTile tile;
     __shared__ double sh[kTileThreads / 32];
+    grid_wait();
+    grid_release();
     const int b0 = blockIdx.x * kTileRows, c0 = blockIdx.y * kTileCols, cl = threadIdx.x % kTileCols, c = c0 + cl;
     const float scale = (float)B * (float)n_obs;
     float d[kTilePer];
@@ -195,6 +200,8 @@ __global__ void __launch_bounds__(kTileThreads) loss_grad_kernel(const float* Z,
 constexpr int kRowsumThreads = 256;
 __global__ void __launch_bounds__(kRowsumThreads) rowsum_kernel(const __nv_bfloat16* Xt, int B, int ld, float* out) {
     __shared__ float sh[kRowsumThreads / 32];
+    grid_wait();
+    grid_release();
     const __nv_bfloat16* x = Xt + (size_t)blockIdx.x * ld;
     const int B8 = B & ~7;
     float s = 0.0f;
@@ -479,8 +486,8 @@ int Handle::mlp_forward(int level, int B, const double* theta, bool training) {
     Mlp& S = mlps[level];
     RC_CHECK(mlp_work(B));
     const int ldt = mwork.ldt;
-    input_kernel<<<tile_grid(B, S.d[0]), kTileThreads, 0, stream>>>(theta, B, K, S.d[0], mwork.X[0],
-                                                                   training ? mwork.Xt[0] : nullptr, ldt);
+    launch_after(input_kernel, tile_grid(B, S.d[0]), dim3(kTileThreads), 0, stream, theta, B, K, S.d[0], mwork.X[0],
+                 training ? mwork.Xt[0] : nullptr, ldt);
     count_launches(1);
     for (int l = 0; l < 5; ++l) {
         GemmEpi epi;
@@ -525,8 +532,8 @@ int Handle::mlp_backward(int level, int B, double* loss) {
     const int NOp = S.d[5];
     const dim3 tiles = tile_grid(B, NOp);
     const int nb = (int)(tiles.x * tiles.y);
-    loss_grad_kernel<<<tiles, kTileThreads, 0, stream>>>(mwork.Z, mwork.tgt, B, NOp, n_obs, mwork.dZ[4], mwork.dZt[4], ldt,
-                                                         mwork.partial);
+    launch_after(loss_grad_kernel, tiles, dim3(kTileThreads), 0, stream, mwork.Z, mwork.tgt, B, NOp, n_obs, mwork.dZ[4],
+                 mwork.dZt[4], ldt, mwork.partial);
     count_launches(1);
     for (int l = 4; l >= 0; --l) {
         // weight gradient dW_l = dZ_l^T X_l  (M = out, N = in, K = batch)
@@ -538,7 +545,7 @@ int Handle::mlp_backward(int level, int B, double* loss) {
         ew.ws_floats = mwork.splitk_floats;
         cudaError_t e = umma_gemm(mwork.dZt[l], ldt, mwork.Xt[l], ldt, S.d[l + 1], S.d[l], B, ew, S.err, stream);
         if (e != cudaSuccess) return cuda_fail(e, "surrogate weight-gradient GEMM");
-        rowsum_kernel<<<S.d[l + 1], kRowsumThreads, 0, stream>>>(mwork.dZt[l], B, ldt, S.gb[l]);
+        launch_after(rowsum_kernel, dim3(S.d[l + 1]), dim3(kRowsumThreads), 0, stream, mwork.dZt[l], B, ldt, S.gb[l]);
         count_launches(1);
         if (l > 0) {
             // input gradient through the GELU of layer l-1: dZ_{l-1} = (dZ_l W_l) * GELU'(pre_{l-1})

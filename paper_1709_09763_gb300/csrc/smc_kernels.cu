@@ -15,6 +15,7 @@
 #include <cstdint>
 
 #include "handle.h"
+#include "launch.h"
 #include "smc_device.h"
 
 namespace mls2mc {
@@ -102,6 +103,8 @@ constexpr int kNormThreads = 64;
 __global__ void __launch_bounds__(kNormThreads) normals_kernel(double* out, int J, int K, uint32_t event, uint32_t purpose, uint64_t seed,
                                const double* base, double c0, double c1) {
     // out[j][k] = c0 * base[j][k] + c1 * xi[j][k]  (base == null: out = xi)
+    grid_wait();
+    grid_release();
     const int nb = (K + 1) / 2;
     const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= (long long)J * nb) return;
@@ -780,6 +783,8 @@ __global__ void __launch_bounds__(kAccThreads) pcn_accept_kernel(
     int n, int K, double beta, const double* beta_p, double zeta, const double* zeta_p, uint32_t event, uint64_t seed,
     double* theta, const double* theta_p, double* phi_c, const double* phi_cp, double* phi_f, const double* phi_fp,
     unsigned long long* n_acc, int rwm) {
+    grid_wait();
+    grid_release();
     if (beta_p) beta = *beta_p;
     if (zeta_p) zeta = *zeta_p;
     pcn_accept_rows((int)blockIdx.x * kAccRows, n, K, beta, zeta, event, seed, theta, theta_p, phi_c, phi_cp, phi_f,
@@ -1042,9 +1047,10 @@ cudaError_t normals_launch(double* out, int J, int K, uint32_t event, uint32_t p
                            const double* base, double c0, double c1, cudaStream_t st) {
     if (J <= 0) return cudaSuccess;
     const long long work = (long long)J * ((K + 1) / 2);
-    normals_kernel<<<grid_for(work, kNormThreads), kNormThreads, 0, st>>>(out, J, K, event, purpose, seed, base, c0, c1);
+    const cudaError_t e = launch_after(normals_kernel, dim3(grid_for(work, kNormThreads)), dim3(kNormThreads), 0, st, out, J, K,
+                                       event, purpose, seed, base, c0, c1);
     count_launches(1);
-    return cudaGetLastError();
+    return e != cudaSuccess ? e : cudaGetLastError();
 }
 
 cudaError_t uniforms_launch(double* out, int J, uint32_t event, uint32_t purpose, uint64_t seed, cudaStream_t st) {
@@ -1117,10 +1123,11 @@ cudaError_t pcn_accept_launch(int n, int K, double beta, const double* beta_p, d
                               const double* phi_cp, double* phi_f, const double* phi_fp, unsigned long long* n_acc,
                               int rwm, cudaStream_t st) {
     if (n <= 0) return cudaSuccess;
-    pcn_accept_kernel<<<grid_for(n, kAccRows), kAccThreads, 0, st>>>(n, K, beta, beta_p, zeta, zeta_p, event, seed, theta, theta_p,
-                                                      phi_c, phi_cp, phi_f, phi_fp, n_acc, rwm);
+    const cudaError_t e = launch_after(pcn_accept_kernel, dim3(grid_for(n, kAccRows)), dim3(kAccThreads), 0, st, n, K, beta,
+                                       beta_p, zeta, zeta_p, event, seed, theta, theta_p, phi_c, phi_cp, phi_f, phi_fp,
+                                       n_acc, rwm);
     count_launches(1);
-    return cudaGetLastError();
+    return e != cudaSuccess ? e : cudaGetLastError();
 }
 
 cudaError_t da_stage1_launch(int n, int K, double beta, double zeta, uint32_t event, uint64_t seed, const double* ps_c,

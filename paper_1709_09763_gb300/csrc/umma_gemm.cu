@@ -25,6 +25,7 @@
 #include <unordered_map>
 
 #include "internal.h"
+#include "launch.h"
 #include "umma_gemm.h"
 
 namespace mls2mc {
@@ -184,7 +185,9 @@ umma_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    grid_wait();   // barriers and tensor memory are set up while the predecessor ends
     __syncthreads();
+    grid_release();
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const uint32_t tmem = tmem_slot;
 
@@ -353,6 +356,8 @@ umma_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
 constexpr int kReduceThreads = 128;
 __global__ void __launch_bounds__(kReduceThreads) splitk_reduce_kernel(const float* ws, int splits, int M, int N, int ld,
                                                                        float* out) {
+    grid_wait();
+    grid_release();
     const int c = blockIdx.x * blockDim.x + threadIdx.x;
     if (c >= N) return;
     const size_t i = (size_t)blockIdx.y * ld + c, slice = (size_t)M * ld;
@@ -455,9 +460,9 @@ cudaError_t launch_gemm(const CUtensorMap& ta, const CUtensorMap& tb, const CUte
         attr_set.fetch_or(bit);
     }
     dim3 grid((N + BN - 1) / BN, (M + BM - 1) / BM, splits);
-    kern<<<grid, 128, smem, st>>>(ta, tb, tc, M, N, K, cps, epi, err);
+    const cudaError_t e = launch_after(kern, grid, dim3(128), smem, st, ta, tb, tc, M, N, K, cps, epi, err);
     count_launches(1);
-    return cudaGetLastError();
+    return e != cudaSuccess ? e : cudaGetLastError();
 }
 
 }  // namespace
@@ -504,10 +509,10 @@ cudaError_t umma_gemm(const void* A, int lda, const void* B, int ldb, int M, int
                                  : launch_gemm<128, 2>(ta, tb, tc, M, N, K, splits, cps, e2, err, st);
         if (e != cudaSuccess) return e;
         const int threads = std::min(kReduceThreads, (N + 31) / 32 * 32);   // M < 38 tiles of 128 rows
-        splitk_reduce_kernel<<<dim3((N + threads - 1) / threads, M), threads, 0, st>>>(epi.ws, splits, M, N, epi.ld_out,
-                                                                                      epi.out_f32);
+        e = launch_after(splitk_reduce_kernel, dim3((N + threads - 1) / threads, M), dim3(threads), 0, st, epi.ws, splits, M,
+                         N, epi.ld_out, epi.out_f32);
         count_launches(1);
-        return cudaGetLastError();
+        return e != cudaSuccess ? e : cudaGetLastError();
     }
     // FP32 outputs without a bias (the KL synthesis) leave by TMA stores when their map encodes
     if ((epi.kind == kEpiExp || (epi.kind == kEpiStoreF32 && !epi.bias)) && cached_map(&tc, epi.out_f32, M, N, epi.ld_out, -1))
