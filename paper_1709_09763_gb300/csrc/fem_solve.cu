@@ -1239,6 +1239,7 @@ fem_eval_kernel(FemArgs a) {
 template <typename Real, int N, int T>
 __global__ void __launch_bounds__(T, (solve_min_blocks<Real, N, T>()))
 fem_eval_kernel_fc(FemArgs a) {
+    grid_wait();
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ double red_buf[2][64];
     __shared__ Real theta_s[256];
@@ -1298,9 +1299,9 @@ cudaError_t launch_one_fc(const FemArgs& a, cudaStream_t st) {
     auto kern = fem_eval_kernel_fc<Real, N, T>;
     cudaError_t err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (err != cudaSuccess) return err;
-    kern<<<a.n, T, smem, st>>>(a);
+    err = launch_after(kern, dim3(a.n), dim3(T), smem, st, a);
     count_launches(1);
-    return cudaGetLastError();
+    return err != cudaSuccess ? err : cudaGetLastError();
 }
 
 template <typename Real, int N, int T>
