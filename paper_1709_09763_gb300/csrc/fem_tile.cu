@@ -27,7 +27,7 @@
 // fem_solve.cu) a node update reads nine words from shared memory, 21 block barriers an iteration; that
 // form (two 512-thread blocks an SM on 1/64) took 1.99 ms for 4000 particles on 1/64 and 0.42 ms on
 // 1/32. Here a patch of 16 nodes reads 8 rim words per half sweep, 17 barriers an iteration, 256 threads
-// of 128 registers, two blocks an SM (1/64) or 64 threads, eight blocks (1/32): 0.76 ms and 0.16 ms. On
+// of 128 registers, two blocks an SM (1/64) or 64 threads, eight blocks (1/32): 0.77 ms and 0.17 ms. On
 // 1/128 (8000 particles) one node per slot on two CTAs of 1024 threads took 31.5 ms, this form 13.1 ms; on
 // 1/256 (1001 particles) the fine levels in device memory took 34.2 ms, this form 12.7 ms.
 // What bounds it is latency: one 1/64 particle alone on an SM takes 0.87 of the time that two take
@@ -56,6 +56,10 @@ struct Geo {
     static constexpr int N = N_, C = C_, TX = N / 4;
     static constexpr bool H = C > 1;
     static constexpr int R = N / 4 / C;
+    // whether a launch may overlap its predecessor's end (launch.h). 4000 particles on 1/32 190 -> 183 us (with the
+    // overlap of the kernels before) and 1001 on 1/256 13.02 -> 12.93 ms; on 1/64 and 1/128 the overlapped
+    // launch came out slower, 4000 particles 808 -> 817 us and 8000 13.37 -> 13.51 ms, so those are plain
+    static constexpr bool OVERLAP = N == 32 || N == 256;
     static constexpr int T = TX * R, NW = T / 32;
     static constexpr bool L2 = N == 256;         // a distributed one-node-per-thread level (1/64)
     static constexpr int TOP = L2 ? N / 8 : N / 4;   // finest level that every CTA solves as a whole
@@ -1027,7 +1031,7 @@ __global__ void __launch_bounds__(G::T, G::MINB) fem_tile_kernel(FemArgs a, floa
     __shared__ int item_s[2];
     const int rank = G::H ? cluster_rank() : 0;
     float4* ref = ref_scratch + (size_t)blockIdx.x * G::REF4;
-    grid_wait();
+    if constexpr (G::OVERLAP) grid_wait();
     const int last = a.n + (int)gridDim.x / G::C - 1;
     auto take = [&](int k) {
         const int item = atomicAdd(counter, 1);
@@ -1133,7 +1137,7 @@ cudaError_t launch_one(const FemArgs& a, float* ref_scratch, int grid, int* coun
     cudaLaunchConfig_t cfg;
     cudaLaunchAttribute attr[2];
     config<G>(cfg, attr[0], grid, st);
-    if (may_overlap(st)) overlap_attr(attr[cfg.numAttrs++]);
+    if (G::OVERLAP && may_overlap(st)) overlap_attr(attr[cfg.numAttrs++]);
     e = cudaLaunchKernelEx(&cfg, fem_tile_kernel<G, RHS>, a, reinterpret_cast<float4*>(ref_scratch), counter);
     count_launches(1);
     return e != cudaSuccess ? e : cudaGetLastError();
