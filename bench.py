@@ -34,16 +34,19 @@ import numpy as np  # noqa: E402
 WORKLOAD = "mls2mc_mixed_h8_64"
 
 
-# DRAM bytes per particle of the 1/64 solve kernels by threads per particle (kappa in, G and Phi
-# out), measured with ncu (dram__bytes_read.sum + dram__bytes_write.sum) on one launch of the same
-# kernel and scaled by the particle count (the traffic is per particle: nothing is shared between
-# blocks); None where no capture of the current build exists
-FEM64_DRAM_BYTES_PER_PARTICLE = {512: None, 1024: None, -512: (20.061184e6 + 4.715776e6) / 608}
+# Per particle of the 1/64 solve kernel, measured with ncu on one launch of 608 particles and scaled by the
+# particle count (nothing is shared between blocks): DRAM bytes (dram__bytes_read.sum +
+# dram__bytes_write.sum: kappa in, G and Phi out) and shared-memory wavefronts of 128 bytes
+# (l1tex__data_pipe_lsu_wavefronts_mem_shared.sum)
+FEM64_DRAM_BYTES_PER_PARTICLE = 20.003328e6 / 608
+FEM64_SMEM_WAVEFRONTS_PER_PARTICLE = 20.431888e6 / 608
 
 
 def solve_kernel_name(N, T):
-    """Name of the solve kernel that runs level 1/h = N with T threads per particle."""
-    return f"fem_eval_compact<{N},{-T}>" if T < 0 else f"fem_eval_kernel<float,{N},{T}>"
+    """Name of the mixed-precision solve kernel that runs level 1/h = N with block size T."""
+    if N >= 32 and (N, T) != (128, 1024):
+        return f"fem_tile_kernel<{N}>"
+    return f"fem_eval_global<{N}>" if N >= 128 else f"fem_eval_kernel<float,{N},{T}>"
 
 
 def algorithmic_flops_per_eval(N, K, iters, passes, synthesis=False):
@@ -64,8 +67,9 @@ def algorithmic_flops_per_eval(N, K, iters, passes, synthesis=False):
 
 
 def algorithmic_smem_bytes_per_eval(N, iters, passes):
-    """Shared-memory bytes one evaluation on level 1/h = N moves, counted from the solve's algorithm
-    (4-byte words; the block reductions' broadcast reads are not counted).
+    """Shared-memory bytes one evaluation on level 1/h = N moves in the one-node-per-slot form, counted from the
+    solve's algorithm (4-byte words; the block reductions' broadcast reads are not counted). The register-tiled
+    form (1/32 and finer) moves fewer: its figure is measured.
 
     Per fine node and CG iteration: a black node loads 9 words (4 weights, 4 neighbours, its inverse
     diagonal) and stores 1 in the black pre-sweep, loads 13 (the same plus 4 coarse values) and
@@ -853,11 +857,11 @@ def main():
         mean_it = float(it.mean())
         kl = L - 1
         launch_ms = kern_ms[kl] / max(kern_n[kl], 1)
-        per_particle = FEM64_DRAM_BYTES_PER_PARTICLE.get(tuned[-1]) if w.inv_h[-1] == 64 else None
-        traffic = per_particle * J if per_particle is not None else None
+        traffic = FEM64_DRAM_BYTES_PER_PARTICLE * J if w.inv_h[-1] == 64 else None
         flops = algorithmic_flops_per_eval(w.inv_h[-1], w.K, mean_it, 2.0) * J
         achieved = flops / (launch_ms * 1e-3) / 1e12
-        smem_tbs = algorithmic_smem_bytes_per_eval(w.inv_h[-1], mean_it, 2.0) * J / (launch_ms * 1e-3) / 1e12
+        smem_tbs = (FEM64_SMEM_WAVEFRONTS_PER_PARTICLE * 128 * J / (launch_ms * 1e-3) / 1e12
+                    if w.inv_h[-1] == 64 else None)
         smem_peak = 152 * 128 * sm_mhz * 1e6 / 1e12           # TB/s, one 128-byte wavefront per SM cycle
         total_evals = evals_per_step * world
         line = {
@@ -880,8 +884,9 @@ def main():
                                    "solve_kernel": solve_kernel_name(N, tuned[l]),
                                    # shared-memory roofline of the level's solve (mean CG iterations
                                    # of the finest level stand in for every level: 10-12 measured)
+                                   # (one-node-per-slot forms only; the finest level's is roofline_smem)
                                    "smem_frac": algorithmic_smem_bytes_per_eval(N, mean_it, 2.0) * J /
-                                   (kern_ms[l] / max(kern_n[l], 1) * 1e-3) / 1e12 / smem_peak}
+                                   (kern_ms[l] / max(kern_n[l], 1) * 1e-3) / 1e12 / smem_peak if N < 32 else None}
                           for l, (N, lm) in enumerate(zip(w.inv_h, lvl_ms))},
             "roofline": {"kernel": solve_kernel_name(w.inv_h[-1], tuned[-1]), "bound": "alu",
                          "achieved": achieved, "peak": fp32_peak, "unit": "TFLOP/s",
@@ -891,11 +896,11 @@ def main():
                          "launches": kern_n[kl], "mean_cg_iters": mean_it,
                          "peak_source": f"FP32 FMA issue rate: 152 SMs x 128 lanes x 2 x {sm_mhz:.0f} MHz "
                                         f"(sm_max_mhz {src})"},
-            # the bound that holds the solve: the shared-memory pipe (the FP32 issue roofline above
-            # is the contract's "alu" figure; the solve runs on chip, far from both HBM and ALU)
+            # the solve runs on chip, far from HBM and (above) from the FP32 issue rate; the pipe it uses
+            # most is shared memory (wavefronts measured by ncu)
             "roofline_smem": {"kernel": solve_kernel_name(w.inv_h[-1], tuned[-1]), "bound": "smem",
                               "achieved": smem_tbs, "peak": smem_peak, "unit": "TB/s",
-                              "frac": smem_tbs / smem_peak,
+                              "frac": smem_tbs / smem_peak if smem_tbs is not None else None,
                               "peak_source": f"152 SMs x 128 B per cycle x {sm_mhz:.0f} MHz"},
             "e2e": {"value": job_throughput(e2e_evals, world, e2e), "unit": "evals/s",
                     "h2d_bytes_per_step": J * w.K * 8, "d2h_bytes_per_step": J * (w.K + 1) * 8},

@@ -5,8 +5,7 @@ python -m paper_1709_09763_gb300.profile_case [--inv-h 64] [--J 304] [--launches
                                              [--train-steps 0 --batch 8192]
 Uses a workload's KL settings (terms, covariance), source, boundary conditions, observation grid
 and data with seeded particles (default: the MLS^2MC workload); --block forces the threads per
-particle (0: the library default; -512 at 1/h = 64: the compact form; -1024 at 1/h = 128: the
-two-CTA form). --train-steps S instead runs S surrogate Adam steps (after three untimed ones) on
+particle (0: the library default; 1024 at 1/h = 128: the device-memory form). --train-steps S instead runs S surrogate Adam steps (after three untimed ones) on
 minibatches of --batch pairs drawn from 40,000 seeded pairs, with the workload's K and
 observation count, and prints the wall time per step.
 """
