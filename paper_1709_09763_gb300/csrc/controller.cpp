@@ -205,7 +205,7 @@ int Handle::read_counters(unsigned long long* acc, IncState* pending) {
 // buy over the work known so far: a level the sampler passes through with little work never pays
 // for a network, one it stays on pays a bounded multiple of the best choice in hindsight). The
 // first round is estimated as its Adam steps times kDaTrainStepPasses forward passes of the
-// minibatch (one step measured 0.30 ms against about 0.075 ms for a forward pass of 8000 rows at
+// minibatch (when it was set, one step measured 0.30 ms against about 0.075 ms for a forward pass of 8000 rows at
 // K = 64).
 constexpr double kDaCostRatio = 8.0;
 constexpr double kDaAmortize = 2.0;
