@@ -1021,7 +1021,9 @@ __device__ __forceinline__ void solve_tile(const FemArgs& a, const int item, flo
 }
 
 // persistent blocks (clusters: rank 0 hands the ticket to the others) take particles from a ticket
-// counter; the barrier at the end of a solve keeps every CTA from overwriting memory another still reads.
+// counter; the barrier at the end of a solve keeps every CTA from overwriting memory another still reads,
+// and one at the start of a cluster's CTAs (660 cycles a launch) lets rank 0 hand out the first ticket: a
+// CTA's shared memory may be written by others only once it has started, which co-scheduling does not give.
 // Every block (cluster) draws tickets until one lies past the particles, so n + clusters are drawn in
 // all: whoever draws the last returns the counter to 0 for the next launch, which needs no memset.
 template <class G, bool RHS>
@@ -1031,6 +1033,7 @@ __global__ void __launch_bounds__(G::T, G::MINB) fem_tile_kernel(FemArgs a, floa
     __shared__ int item_s[2];
     const int rank = G::H ? cluster_rank() : 0;
     float4* ref = ref_scratch + (size_t)blockIdx.x * G::REF4;
+    if constexpr (G::H) sync_all<G::C>();   // every CTA of the cluster runs before the first store into another's memory
     if constexpr (G::OVERLAP) grid_wait();
     const int last = a.n + (int)gridDim.x / G::C - 1;
     auto take = [&](int k) {
@@ -1062,6 +1065,7 @@ __global__ void __launch_bounds__(G::T, G::MINB)
     __shared__ FemArgs args_s;
     const int rank = G::H ? cluster_rank() : 0;
     float4* ref = ref_scratch + (size_t)blockIdx.x * G::REF4;
+    if constexpr (G::H) sync_all<G::C>();   // as above
     auto take = [&](int k) {
         const int item = atomicAdd(counter, 1);
         item_s[k] = item;
