@@ -228,7 +228,8 @@ umma_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
     __syncwarp();
 
     // epilogue: warp w owns TMEM lanes (tile rows) 32w .. 32w + 31
-    const bool done = mbar_wait(smem_u32(&done_bar), 0);
+    // (the vote brings the lanes together again: tensor memory is read by whole warps, .sync.aligned)
+    const bool done = __all_sync(0xffffffffu, mbar_wait(smem_u32(&done_bar), 0));
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     if (done) {
         const uint32_t t_row = tmem + ((uint32_t)(32 * warp) << 16);
@@ -293,6 +294,8 @@ umma_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
             // backward per 8192 x 256 x 256 product, now 11 and 12 us.)
             const int row = m0 + 32 * warp + lane;
             const bool in = row < M;
+            // rows past the end read the last one: a branch here could leave the warp apart at tmem_ld32
+            const float* pre_in = epi.kind == kEpiGeluBackward ? epi.pre_in + (size_t)min(row, M - 1) * epi.ld_pre : nullptr;
 #pragma unroll 1
             for (int c0 = 0; c0 < BN && n0 + c0 < N; c0 += 32) {
                 const int col = n0 + c0;
@@ -300,12 +303,9 @@ umma_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
                 if (epi.kind == kEpiBiasGelu) {
 #pragma unroll
                     for (int i = 0; i < 32; i += 8) ld_v8(epi.bias + col + i, x + i);
-                } else if (in) {
-#pragma unroll
-                    for (int i = 0; i < 32; i += 8) ld_v8(epi.pre_in + (size_t)row * epi.ld_pre + col + i, x + i);
                 } else {
 #pragma unroll
-                    for (int i = 0; i < 32; ++i) x[i] = 0.0f;
+                    for (int i = 0; i < 32; i += 8) ld_v8(pre_in + col + i, x + i);
                 }
                 tmem_ld32(t_row + (uint32_t)c0, v);
                 if (epi.kind == kEpiBiasGelu) {
