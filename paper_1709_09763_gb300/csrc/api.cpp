@@ -183,7 +183,7 @@ int Handle::eval_device(int level, int n, const double* theta, double* G, double
     } else {
         FemArgs a = fem_args(level, n, theta, G, Phi, iters);
         if (precision == SMC_MIXED) {
-            int rc = synth_kappa(level, n, theta, st);
+            int rc = synth_kappa(level, n, theta, st, true, tile_counter);
             if (rc != SMC_OK) return rc;
             a.kappa = synth_kappa_buf;
         }
@@ -200,11 +200,6 @@ int Handle::eval_device(int level, int n, const double* theta, double* G, double
                 cudaError_t ea = cudaMalloc((void**)&cp_scratch, need * sizeof(float));
                 if (ea != cudaSuccess) return fail(SMC_ENOMEM, "tile-form scratch: %s", cudaGetErrorString(ea));
                 cp_cap = need;
-            }
-            if (!tile_counter) {   // zeroed once: every launch leaves it at 0
-                if (cudaMalloc((void**)&tile_counter, sizeof(int)) != cudaSuccess)
-                    return fail(SMC_ENOMEM, "work counter");
-                cudaMemsetAsync(tile_counter, 0, sizeof(int), st);
             }
             a.bad = bad;   // counted by the solve itself
             bad = nullptr;
@@ -334,6 +329,9 @@ int smc_init(const smc_problem_desc* P, const smc_sampler_opts* O, smc_handle** 
     h->y_host.assign(P->y, P->y + P->n_obs);
     cudaError_t e = upload(&h->d_y, P->y, (size_t)P->n_obs);
     if (e != cudaSuccess) return bail(h->cuda_fail(e, "upload y"));
+    if (P->forward_kind == SMC_FWD_FEM && O->precision == SMC_MIXED &&
+        cudaMalloc((void**)&h->tile_counter, sizeof(int)) != cudaSuccess)
+        return bail(h->fail(SMC_ENOMEM, "work counter"));
     for (int l = 0; l < P->n_levels; ++l) {
         Level L;
         if (P->forward_kind == SMC_FWD_FEM) {

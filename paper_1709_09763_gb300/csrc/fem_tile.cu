@@ -1024,8 +1024,8 @@ __device__ __forceinline__ void solve_tile(const FemArgs& a, const int item, flo
 // counter; the barrier at the end of a solve keeps every CTA from overwriting memory another still reads,
 // and one at the start of a cluster's CTAs (660 cycles a launch) lets rank 0 hand out the first ticket: a
 // CTA's shared memory may be written by others only once it has started, which co-scheduling does not give.
-// Every block (cluster) draws tickets until one lies past the particles, so n + clusters are drawn in
-// all: whoever draws the last returns the counter to 0 for the next launch, which needs no memset.
+// Every block (cluster) draws tickets until one lies past the particles. The counter is 0 before each launch:
+// the split of theta that starts the evaluation zeroes it (a memset of its own would be one more launch).
 template <class G, bool RHS>
 __global__ void __launch_bounds__(G::T, G::MINB) fem_tile_kernel(FemArgs a, float4* ref_scratch, int* counter) {
     extern __shared__ __align__(16) float sm[];
@@ -1035,10 +1035,8 @@ __global__ void __launch_bounds__(G::T, G::MINB) fem_tile_kernel(FemArgs a, floa
     float4* ref = ref_scratch + (size_t)blockIdx.x * G::REF4;
     if constexpr (G::H) sync_all<G::C>();   // every CTA of the cluster runs before the first store into another's memory
     if constexpr (G::OVERLAP) grid_wait();
-    const int last = a.n + (int)gridDim.x / G::C - 1;
     auto take = [&](int k) {
         const int item = atomicAdd(counter, 1);
-        if (item == last) *counter = 0;
         item_s[k] = item;
         if constexpr (G::H)
             for (int c = 1; c < G::C; ++c) st_peer(&item_s[k], c, item);

@@ -58,7 +58,7 @@ struct Handle {
     size_t cp_cap = 0;
     size_t big_cap = 0;
     int* big_counter = nullptr;
-    int* tile_counter = nullptr;   // ticket of the register-tiled form: 0 between launches
+    int* tile_counter = nullptr;   // ticket of the register-tiled form (mixed path; made by smc_init)
 
     // tensor-core KL synthesis buffers (kl_synth.cu)
     float* synth_kappa_buf = nullptr;
@@ -67,8 +67,9 @@ struct Handle {
     float* synth_part_buf = nullptr;   // K > 256: FP32 partial fields of the term groups [groups][n][E]
     size_t synth_part_cap = 0;
     int* synth_err = nullptr;
-    // split: false where theta_split_multi_launch has split theta already (one contraction only)
-    int synth_kappa(int level, int n, const double* theta, cudaStream_t st, bool split = true);
+    // split: false where theta_split_multi_launch has split theta already (one contraction only);
+    // ticket (device, with split): set to 0 on the way, for the solve that follows
+    int synth_kappa(int level, int n, const double* theta, cudaStream_t st, bool split = true, int* ticket = nullptr);
     int synth_reserve(int level, int n);
 
     // opt-in CUDA-event timing of forward-solve launches, per level

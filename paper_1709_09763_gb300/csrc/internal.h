@@ -89,8 +89,8 @@ cudaError_t fem_eval_persistent_launch(int N, int precision, int T, const FemArg
 // register-tiled form of the mixed solve (fem_tile.cu): 1/32 and 1/64 on one CTA (every block size of those
 // levels), 1/128 on a cluster of two CTAs (block size -1024), 1/256 of eight; not the flow cell. Where a
 // cluster does not fit, 1/128 and 1/256 run in the device-memory form above. fem_tile_scratch floats of device
-// scratch hold the refinement state. *counter (device) is 0 before a launch; fem_tile_launch leaves it at 0,
-// fem_tile_multi_launch (arguments as fem_eval_persistent_launch) does not
+// scratch hold the refinement state. *counter (device) is 0 before a launch (fem_tile_launch: zeroed by the
+// evaluation's Handle::synth_kappa); fem_tile_multi_launch: arguments as fem_eval_persistent_launch
 bool fem_tile_form(int N, int precision, bool flow_cell);
 size_t fem_tile_scratch(int N);
 cudaError_t fem_tile_launch(const FemArgs& a, float* scratch, int* counter, cudaStream_t st);

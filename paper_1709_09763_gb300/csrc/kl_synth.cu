@@ -78,9 +78,10 @@ __device__ __forceinline__ void split_row(const double* th, int Kg, int Kp, int 
 
 template <int V>
 __global__ void __launch_bounds__(kSplitThreads)
-    theta_split_kernel(const double* theta, int n, int K, int k0, int Kg, int Kp, __nv_bfloat16* out) {
+    theta_split_kernel(const double* theta, int n, int K, int k0, int Kg, int Kp, __nv_bfloat16* out, int* ticket) {
     grid_wait();
     grid_release();
+    if (ticket && blockIdx.x == 0 && threadIdx.x == 0 && threadIdx.y == 0) *ticket = 0;
     const long long j = (long long)blockIdx.x * blockDim.y + threadIdx.y;
     if (j < n)
         split_row<V>(theta + (size_t)j * K + k0, Kg, Kp, (int)threadIdx.x, (int)blockDim.x, out + (size_t)j * Kp);
@@ -100,13 +101,14 @@ __global__ void __launch_bounds__(kSplitThreads) theta_split_multi_kernel(const 
     }
 }
 
-void theta_split_launch(const double* theta, int n, int K, int k0, int Kg, int Kp, __nv_bfloat16* out, cudaStream_t st) {
+void theta_split_launch(const double* theta, int n, int K, int k0, int Kg, int Kp, __nv_bfloat16* out, int* ticket,
+                        cudaStream_t st) {
     const int terms = Kg % 2 == 0 ? Kg / 2 : Kg;
     const int kx = std::min(terms, kSplitThreads), ry = kSplitThreads / kx;
     const dim3 block(kx, ry);
     const unsigned grid = (unsigned)(((long long)n + ry - 1) / ry);
     launch_after(Kg % 2 == 0 ? theta_split_kernel<2> : theta_split_kernel<1>, grid, block, 0, st, theta, n, K, k0, Kg, Kp,
-                 out);
+                 out, ticket);
     count_launches(1);
 }
 
@@ -232,13 +234,13 @@ cudaError_t theta_split_multi_launch(const std::vector<SplitTask>& tasks, cudaSt
     return cudaSuccess;
 }
 
-int Handle::synth_kappa(int level, int n, const double* theta, cudaStream_t st, bool split) {
+int Handle::synth_kappa(int level, int n, const double* theta, cudaStream_t st, bool split, int* ticket) {
     const Level& L = levels[level];
     const int E = 2 * L.N * L.N, Kt = kl_split_total(K), G = kl_groups(K);
     RC_CHECK(synth_reserve(level, n));
     if (G == 1) {
         if (split)
-            theta_split_launch(theta, n, K, 0, K, Kt, reinterpret_cast<__nv_bfloat16*>(synth_theta_buf), st);
+            theta_split_launch(theta, n, K, 0, K, Kt, reinterpret_cast<__nv_bfloat16*>(synth_theta_buf), ticket, st);
         GemmEpi epi;
         epi.kind = kEpiExp;
         epi.out_f32 = synth_kappa_buf;
@@ -251,7 +253,7 @@ int Handle::synth_kappa(int level, int n, const double* theta, cudaStream_t st, 
     for (int g = 0; g < G; ++g) {
         const int Kg = group_terms(K, g), Kp = kl_split_width(Kg);
         theta_split_launch(theta, n, K, g * kSynthGroup, Kg, Kp, reinterpret_cast<__nv_bfloat16*>(synth_theta_buf + off_t),
-                           st);
+                           ticket, st);
         GemmEpi epi;
         epi.kind = kEpiStoreF32;
         epi.out_f32 = synth_part_buf + (size_t)g * n * E;
