@@ -941,18 +941,7 @@ __device__ __forceinline__ void solve_tile(const FemArgs& a, const int item, flo
                 float eh, el, nh, nl;
                 flux(wE[b][i + 1], p[b][i], i < 3 ? p[b][i < 3 ? i + 1 : 3] : hR[b], eh, el);
                 flux(wN[b + 1][i], p[b][i], b < 3 ? p[b < 3 ? b + 1 : 3][i] : hA[i], nh, nl);
-                // r -= (east + north) - (west + south): high parts by TwoSum, the rest in one low part
-                float h = rh[i], l = rl[i], t;
-                two_sum(h, -eh, h, t);
-                l += t - el;
-                two_sum(h, wsh, h, t);
-                l += t + wsl;
-                two_sum(h, -nh, h, t);
-                l += t - nl;
-                two_sum(h, sth[i], h, t);
-                l += t + stl[i];
-                rh[i] = h + l;
-                rl[i] = l - (rh[i] - h);
+                df_residual(rh[i], rl[i], eh, el, -wsh, -wsl, nh, nl, -sth[i], -stl[i]);
                 if (fixed(i, b)) rh[i] = rl[i] = 0.f;
                 rr_out += rh[i] * rh[i];
                 wsh = eh;
