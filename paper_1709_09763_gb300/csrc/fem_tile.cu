@@ -62,6 +62,11 @@ struct Geo {
     static constexpr bool OVERLAP = N == 32 || N == 256;
     static constexpr int T = TX * R, NW = T / 32;
     static constexpr bool L2 = N == 256;         // a distributed one-node-per-thread level (1/64)
+    // the fine inverse diagonals are correctly rounded and in shared memory; on 1/128 there is no room for them and the
+    // sweeps form approximate ones, as that level always has. On 1/256 they take the place of the CG correction d,
+    // which is in device memory there (read and written once an iteration). 1001 particles: 13.53 ms; 12.99 with
+    // approximate ones, 13.98 with them and not d in device memory, 14.97 with a rounded reciprocal in the sweeps
+    static constexpr bool STORED = N != 128, DG = N == 256;
     static constexpr int TOP = L2 ? N / 8 : N / 4;   // finest level that every CTA solves as a whole
     // blocks per SM: registers for 128 a thread
     static constexpr int MINB = 65536 / (128 * T);
@@ -71,11 +76,10 @@ struct Geo {
     // ---- shared memory, in floats ----
     static constexpr int E = 0;              // sweep values, later p or d: rim positions [16][S]; the
                                              // inner positions' slots carry red residuals
-    static constexpr int D = E + 16 * S;     // CG correction d, float4 [4][T]
+    static constexpr int D = E + 16 * S;     // CG correction d, float4 [4][T] (unless DG)
     static constexpr int PV = D + 16 * T;    // CG direction p, float4 [4][T] (not in registers during the V-cycle)
-    // fine inverse diagonals, float4 [red 2, black 2][T]; formed in the sweeps where a cluster has no room
-    static constexpr int ID = PV + 16 * T;
-    static constexpr int W1 = ID + (H ? 0 : 16 * T);  // next level: weights (E, W, N, S) of (0,0) (1,1) (1,0) (0,1)
+    static constexpr int ID = DG ? D : PV + 16 * T;   // fine inverse diagonals, float4 [red 2, black 2][T]
+    static constexpr int W1 = PV + 16 * T + (STORED && !DG ? 16 * T : 0);  // next level: weights (E, W, N, S) of (0,0) (1,1) (1,0) (0,1)
     static constexpr int WH = W1 + 16 * T;   // those of (1,1) in the row of patches below this CTA, float4 [TX]
     static constexpr int E1 = WH + 4 * TX;   // its values [4][S], positions A + 2 B
     // its right-hand side, float4 [T], out of registers while the levels below run on a cluster's CTAs
@@ -105,7 +109,8 @@ struct Geo {
     __host__ __device__ static constexpr int kst(int M) {
         return M == TOP ? (L2 ? D : PV) : M == 16 ? D + (L2 ? 2 * TOP * TOP : 0) : M == 8 ? kst(16) + 512 : kst(16) + 640;
     }
-    static constexpr int REF4 = 16 * T;      // float4s of refinement state of one CTA (device memory)
+    // float4s of refinement state of one CTA (device memory): r hi, r lo, x hi, x lo and, with DG, d
+    static constexpr int REF4 = (DG ? 20 : 16) * T;
     static_assert(FLOATS * 4 <= 226 * 1024, "shared memory of one block");
     static_assert(N != 64 || FLOATS * 4 <= 113 * 1024, "two blocks of 1/64 on an SM");
 };
@@ -377,7 +382,7 @@ __device__ __forceinline__ void solve_tile(const FemArgs& a, const int item, flo
     // exchange-array index of this patch; its neighbours are at q - 1, q + 1, q - TX, q + TX
     const int q = tid + TX, pL = q - 1, pR = q + 1, pB = q - TX, pA = q + TX, pD = pB - 1, pU = pA + 1;
     float* E = sm + G::E;
-    float4* D4 = reinterpret_cast<float4*>(sm + G::D);
+    float4* D4 = G::DG ? ref + 16 * T : reinterpret_cast<float4*>(sm + G::D);
     float4* PV4 = reinterpret_cast<float4*>(sm + G::PV);
     float4* ID4 = reinterpret_cast<float4*>(sm + G::ID);
     float4* W1 = reinterpret_cast<float4*>(sm + G::W1);
@@ -459,10 +464,9 @@ __device__ __forceinline__ void solve_tile(const FemArgs& a, const int item, flo
             }
         }
     }
-    // fine inverse diagonal at node (i, b): one CTA keeps the correctly rounded reciprocal in shared memory; a
-    // cluster forms the approximate one where a sweep needs it (it only shapes the preconditioner)
+    // fine inverse diagonals: 1 / the sum of the edge weights, 0 on Dirichlet nodes
     auto diag = [&](int i, int b) { return wE[b][i + 1] + wE[b][i] + wN[b + 1][i] + wN[b][i]; };
-    if constexpr (!H) {
+    auto store_diag = [&] {
 #pragma unroll
         for (int c = 0; c < 2; ++c)   // colour c, rows 0 1 and rows 2 3
 #pragma unroll
@@ -476,7 +480,8 @@ __device__ __forceinline__ void solve_tile(const FemArgs& a, const int item, flo
                 }
                 ID4[(2 * c + h) * T + tid] = make_float4(v[0], v[1], v[2], v[3]);
             }
-    }
+    };
+    if constexpr (G::STORED && !G::DG) store_diag();
     sync_all<C>();
     {   // next level: the weights of the 2 x 2 nodes
         float lo[3][3], up[3][3];   // cells (-1 .. 1)^2, index [row + 1][column + 1]
@@ -535,6 +540,10 @@ __device__ __forceinline__ void solve_tile(const FemArgs& a, const int item, flo
     }
     if constexpr (H) sync_all<C>();   // the neighbours write into this CTA's arrays only from here on
     levels_setup<G, G::TOP>(sm);
+    if constexpr (G::DG) {   // over the staging that the levels were set up from
+        __syncthreads();
+        store_diag();
+    }
 
     // ---- rim exchange: colour c's values of the neighbouring patches next to the patch's other colour
     float hL[4], hR[4], hB[4], hA[4];
@@ -565,7 +574,7 @@ __device__ __forceinline__ void solve_tile(const FemArgs& a, const int item, flo
                wN[b + 1][i] * (b < 3 ? v[b < 3 ? b + 1 : 3][i] : hA[i]) + wN[b][i] * (b > 0 ? v[b > 0 ? b - 1 : 0][i] : hB[i]);
     };
     auto inv_diag = [&](int c, float (&v)[8]) {   // this thread's inverse diagonals of colour c, in node order
-        if constexpr (!H) {
+        if constexpr (G::STORED) {
             const float4 x = ID4[2 * c * T + tid], y = ID4[(2 * c + 1) * T + tid];
             v[0] = x.x; v[1] = x.y; v[2] = x.z; v[3] = x.w;
             v[4] = y.x; v[5] = y.y; v[6] = y.z; v[7] = y.w;
