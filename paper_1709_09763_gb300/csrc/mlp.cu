@@ -136,11 +136,11 @@ __global__ void sample_indices_kernel(int* idx, int B, int count, uint32_t step,
 // batch_kernel
 __global__ void __launch_bounds__(kTileThreads) targets_kernel(const double* G, int B, int n_obs, int NOp, const float* mu,
                                                                const float* sd, float* tgt) {
-    // FP64 in, FP32 out. Bound by the FP64 instructions: the reciprocal of a column's sd is formed once for
-    // the thread's eight rows (8192 x 49: 14.2 us with a division per element, now 8.1 us)
+    // FP64 in, FP32 out. Bound by the FP64 divisions (a reciprocal per column instead takes a few us less of
+    // 8192 x 49, but rounds some targets the other way)
     const int c = blockIdx.y * kTileCols + threadIdx.x % kTileCols;
     if (c >= NOp) return;
-    const double m = c < n_obs ? (double)mu[c] : 0.0, inv = c < n_obs ? 1.0 / (double)sd[c] : 0.0;
+    const double m = c < n_obs ? (double)mu[c] : 0.0, s = c < n_obs ? (double)sd[c] : 1.0;
     double x[kTilePer];
 #pragma unroll
     for (int i = 0; i < kTilePer; ++i) {
@@ -150,7 +150,7 @@ __global__ void __launch_bounds__(kTileThreads) targets_kernel(const double* G, 
 #pragma unroll
     for (int i = 0; i < kTilePer; ++i) {
         const int b = blockIdx.x * kTileRows + threadIdx.x / kTileCols + i * (kTileThreads / kTileCols);
-        if (b < B) tgt[(size_t)b * NOp + c] = c < n_obs ? (float)((x[i] - m) * inv) : 0.0f;
+        if (b < B) tgt[(size_t)b * NOp + c] = c < n_obs ? (float)((x[i] - m) / s) : 0.0f;
     }
 }
 
