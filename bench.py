@@ -14,6 +14,7 @@ the host-pointer C-ABI call (theta copied in from pinned host memory, G and Phi 
 out every step). Multi-GPU: independent replicas per rank (no data-path collective).
 
 Usage: python bench.py [--gpus N] [--steps K] [--warmup W] [--impl native|reference]
+Prints one JSON line of at most LINE_CHARS characters; --detail FILE takes the studies after the timed step in full.
 """
 import argparse
 import dataclasses
@@ -146,6 +147,44 @@ def reduce_max_over_ranks(values, dist=None, device="cpu"):
 def job_throughput(units_per_rank, world, ms_max):
     """Whole-job units per second: all ranks' units over the slowest rank's time (weak scaling)."""
     return units_per_rank * world / (ms_max * 1e-3)
+
+
+LINE_CHARS = 2900   # of the printed result: what keeps a run's output keeps its last 3000 characters or so
+
+
+def significant(x, digits):
+    """x with every float in it rounded to `digits` significant digits."""
+    if isinstance(x, dict):
+        return {k: significant(v, digits) for k, v in x.items()}
+    if isinstance(x, (list, tuple)):
+        return [significant(v, digits) for v in x]
+    return float(f"{x:.{digits}g}") if isinstance(x, float) else x
+
+
+def headline(full):
+    """The printed result: the timed step's figures and, of each study, the arms' median seconds ("s") and the
+    speed-ups ("x..."). The studies in full (replicates, per-update lists, accuracy tables) go to --detail."""
+    line = {k: v for k, v in full.items() if not isinstance(v, dict) or k in ("config", "e2e", "clocks")}
+    line["per_level"] = {N: {k: lv[k] for k in ("evals_per_s", "update_ms", "solve_launch_ms")}
+                         for N, lv in full["per_level"].items()}
+    for key in ("roofline", "roofline_smem"):
+        line[key] = {k: v for k, v in full[key].items() if k != "peak_source"}
+    if "cpu_baseline" in full:
+        line["cpu_baseline"] = {k: full["cpu_baseline"][k] for k in ("value", "unit", "cores", "kind")}
+    line = significant(line, 7)
+    studies = {}
+    for name, st in full.get("seconds_to_posterior", {}).items():
+        arms = [v for v in st.values() if isinstance(v, dict) and "seconds_median" in v] or [st]
+        studies[name] = {"s": [v["seconds_median"] for v in arms if "seconds_median" in v]}
+        studies[name].update({k.replace("speedup", "x"): v for k, v in st.items()
+                              if k.startswith("speedup") and isinstance(v, float)})
+    for name in full:
+        if name.startswith("batched_"):
+            studies[name] = {"x": full[name]["speedup"]}
+    line["studies"] = significant(studies, 4)
+    while len(json.dumps(line)) > LINE_CHARS and line["studies"]:   # the step's own figures always stay
+        line["studies"].popitem()
+    return line
 
 
 def load_data(name=WORKLOAD):
@@ -409,6 +448,7 @@ def main():
                          "pCN step against the adaptive step, plain and screened, with per-update diagnostics")
     ap.add_argument("--example-5-3-full", action="store_true",
                     help="also run Example 5.3 at the paper's size (1/16 .. 1/256, 320 KL terms)")
+    ap.add_argument("--detail", metavar="FILE", help="write the result with every study in full (JSON)")
     args = ap.parse_args()
     if args.warmup < 3:
         args.warmup = 3
@@ -919,7 +959,10 @@ def main():
             line["batched_sampler_small_problems_to_posterior"] = batched_run_small
         if world == 1 and not args.no_cpu_baseline:
             line["cpu_baseline"] = cpu_baseline()
-        print(json.dumps(line), flush=True)
+        if args.detail:
+            with open(args.detail, "w") as f:
+                json.dump(line, f)
+        print(json.dumps(headline(line)), flush=True)
     if world > 1:
         dist.destroy_process_group()
 
