@@ -180,8 +180,8 @@ int smc_kl_table_host(int cov_kind, int N, double corr_len, double variance, int
  * launches, returns the summed device milliseconds and launch counts per level ([8] arrays,
  * either may be NULL) and forgets them. */
 int smc_set_timing(smc_handle* h, int enable);
-/* Autotuner of the solve kernel (no counterpart in the paper): for every level, time each compiled
- * block size (threads per particle) on n_tune prior draws and keep the fastest for the process
+/* Autotuner of the solve kernel (no counterpart in the paper): for every level, time each block size
+ * that is a kernel of its own on n_tune prior draws and keep the fastest for the process
  * (shared by all handles of the same 1/h and precision). chosen [n_levels] receives the block
  * sizes, best_ms [n_levels] the time per launch (either may be NULL). smc_set_block_size forces a
  * block size for a level (T = 0 restores the default: -512 and -256 on 1/64 and 1/32 of the mixed

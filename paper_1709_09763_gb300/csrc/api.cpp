@@ -481,7 +481,7 @@ int smc_autotune(smc_handle* hh, int n_tune, int* chosen, float* best_ms) {
         const int N = h->levels[l].N;
         int bestT = 0;
         float best = 0.f;
-        for (int T : fem_block_sizes(N, h->precision)) {
+        for (int T : fem_block_forms(N, h->precision)) {
             set_block(N, h->precision, T);
             for (int rep = 0; rep < 4; ++rep) {
                 if (rep == 1) cudaEventRecord(e0, st);

@@ -1439,8 +1439,17 @@ int fem_default_block(int N, int precision) {
     return s.empty() ? 0 : s[0];
 }
 
-// block sizes compiled for each level (threads per particle); the autotuner picks one. FP64: 64 at 1/8 names
-// one warp per particle and 256 at 1/32 four (per-warp work such as the reductions' sums and the divisions
+std::vector<int> fem_block_forms(int N, int precision) {
+    const int T0 = fem_default_block(N, precision);
+    if (T0 == 0 || (precision == SMC_MIXED && (N == 32 || N == 64))) return {T0};   // every size is the same kernel
+    std::vector<int> forms = {T0};
+    for (int T : fem_block_sizes(N, precision))
+        if (T != T0) forms.push_back(T);
+    return forms;
+}
+
+// names of the block sizes of each level; on the mixed path up to 1/16 and in FP64 threads per particle, but for
+// FP64's 64 at 1/8, which names one warp per particle, and 256 at 1/32, four (per-warp work such as the reductions' sums and the divisions
 // is FP64 time: 1000 particles 197 -> 149 us and, with the exact 1/4 level, 2120 -> 1970 us)
 std::vector<int> fem_block_sizes(int N, int precision) {
     if (precision == SMC_MIXED) {
