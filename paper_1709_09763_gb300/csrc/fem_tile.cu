@@ -56,10 +56,6 @@ struct Geo {
     static constexpr int N = N_, C = C_, TX = N / 4;
     static constexpr bool H = C > 1;
     static constexpr int R = N / 4 / C;
-    // whether a launch may overlap its predecessor's end (launch.h). 4000 particles on 1/32 190 -> 183 us (with the
-    // overlap of the kernels before) and 1001 on 1/256 13.02 -> 12.93 ms; on 1/64 and 1/128 the overlapped
-    // launch came out slower, 4000 particles 808 -> 817 us and 8000 13.37 -> 13.51 ms, so those are plain
-    static constexpr bool OVERLAP = N == 32 || N == 256;
     static constexpr int T = TX * R, NW = T / 32;
     static constexpr bool L2 = N == 256;         // a distributed one-node-per-thread level (1/64)
     // the fine inverse diagonals are correctly rounded and in shared memory; on 1/128 there is no room for them and the
@@ -1032,7 +1028,7 @@ __global__ void __launch_bounds__(G::T, G::MINB) fem_tile_kernel(FemArgs a, floa
     const int rank = G::H ? cluster_rank() : 0;
     float4* ref = ref_scratch + (size_t)blockIdx.x * G::REF4;
     if constexpr (G::H) sync_all<G::C>();   // every CTA of the cluster runs before the first store into another's memory
-    if constexpr (G::OVERLAP) grid_wait();
+    grid_wait();
     auto take = [&](int k) {
         const int item = atomicAdd(counter, 1);
         item_s[k] = item;
@@ -1137,7 +1133,7 @@ cudaError_t launch_one(const FemArgs& a, float* ref_scratch, int grid, int* coun
     cudaLaunchConfig_t cfg;
     cudaLaunchAttribute attr[2];
     config<G>(cfg, attr[0], grid, st);
-    if (G::OVERLAP && may_overlap(st)) overlap_attr(attr[cfg.numAttrs++]);
+    if (may_overlap(st)) overlap_attr(attr[cfg.numAttrs++]);   // launch.h
     e = cudaLaunchKernelEx(&cfg, fem_tile_kernel<G, RHS>, a, reinterpret_cast<float4*>(ref_scratch), counter);
     count_launches(1);
     return e != cudaSuccess ? e : cudaGetLastError();

@@ -80,7 +80,6 @@ template <int V>
 __global__ void __launch_bounds__(kSplitThreads)
     theta_split_kernel(const double* theta, int n, int K, int k0, int Kg, int Kp, __nv_bfloat16* out, int* ticket) {
     grid_wait();
-    grid_release();
     if (ticket && blockIdx.x == 0 && threadIdx.x == 0 && threadIdx.y == 0) *ticket = 0;
     const long long j = (long long)blockIdx.x * blockDim.y + threadIdx.y;
     if (j < n)

@@ -75,7 +75,6 @@ __global__ void __launch_bounds__(kTileThreads) input_kernel(const double* theta
                                                              __nv_bfloat16* Xt, int ldt) {
     __shared__ __align__(16) BatchTile tile;
     grid_wait();
-    grid_release();
     const int b0 = blockIdx.x * kTileRows, c0 = blockIdx.y * kTileCols, cl = threadIdx.x % kTileCols, k = c0 + cl;
     double x[kTilePer];
 #pragma unroll
@@ -164,7 +163,6 @@ __global__ void __launch_bounds__(kTileThreads) loss_grad_kernel(const float* Z,
     __shared__ __align__(16) BatchTile tile;
     __shared__ double sh[kTileThreads / 32];
     grid_wait();
-    grid_release();
     const int b0 = blockIdx.x * kTileRows, c0 = blockIdx.y * kTileCols, cl = threadIdx.x % kTileCols, c = c0 + cl;
     const float scale = (float)B * (float)n_obs;
     float d[kTilePer];
@@ -201,7 +199,6 @@ constexpr int kRowsumThreads = 256;
 __global__ void __launch_bounds__(kRowsumThreads) rowsum_kernel(const __nv_bfloat16* Xt, int B, int ld, float* out) {
     __shared__ float sh[kRowsumThreads / 32];
     grid_wait();
-    grid_release();
     const __nv_bfloat16* x = Xt + (size_t)blockIdx.x * ld;
     const int B8 = B & ~7;
     float s = 0.0f;

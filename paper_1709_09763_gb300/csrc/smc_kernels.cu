@@ -111,7 +111,6 @@ __global__ void __launch_bounds__(kNormThreads) normals_kernel(double* out, int 
                                const double* base, double c0, double c1) {
     // out[j][k] = c0 * base[j][k] + c1 * xi[j][k]  (base == null: out = xi)
     grid_wait();
-    grid_release();
     const int nb = (K + 1) / 2;
     const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= (long long)J * nb) return;
@@ -791,7 +790,6 @@ __global__ void __launch_bounds__(kAccThreads) pcn_accept_kernel(
     double* theta, const double* theta_p, double* phi_c, const double* phi_cp, double* phi_f, const double* phi_fp,
     unsigned long long* n_acc, int rwm) {
     grid_wait();
-    grid_release();
     if (beta_p) beta = *beta_p;
     if (zeta_p) zeta = *zeta_p;
     pcn_accept_rows((int)blockIdx.x * kAccRows, n, K, beta, zeta, event, seed, theta, theta_p, phi_c, phi_cp, phi_f,

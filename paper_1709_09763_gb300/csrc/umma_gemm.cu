@@ -187,7 +187,6 @@ umma_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     grid_wait();   // barriers and tensor memory are set up while the predecessor ends
     __syncthreads();
-    grid_release();
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const uint32_t tmem = tmem_slot;
 
@@ -357,7 +356,6 @@ constexpr int kReduceThreads = 128;
 __global__ void __launch_bounds__(kReduceThreads) splitk_reduce_kernel(const float* ws, int splits, int M, int N, int ld,
                                                                        float* out) {
     grid_wait();
-    grid_release();
     const int c = blockIdx.x * blockDim.x + threadIdx.x;
     if (c >= N) return;
     const size_t i = (size_t)blockIdx.y * ld + c, slice = (size_t)M * ld;
