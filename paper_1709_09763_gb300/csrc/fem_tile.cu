@@ -75,13 +75,15 @@ struct Geo {
     static constexpr int D = E + 16 * S;     // CG correction d, float4 [4][T] (unless DG)
     static constexpr int PV = D + 16 * T;    // CG direction p, float4 [4][T] (not in registers during the V-cycle)
     static constexpr int ID = DG ? D : PV + 16 * T;   // fine inverse diagonals, float4 [red 2, black 2][T]
-    static constexpr int W1 = PV + 16 * T + (STORED && !DG ? 16 * T : 0);  // next level: weights (E, W, N, S) of (0,0) (1,1) (1,0) (0,1)
+    // next level: weights (E, W, N, S) of (0,0) (1,1) (1,0) (0,1)
+    static constexpr int W1 = PV + 16 * T + (STORED && !DG ? 16 * T : 0);
     static constexpr int WH = W1 + 16 * T;   // those of (1,1) in the row of patches below this CTA, float4 [TX]
     static constexpr int E1 = WH + 4 * TX;   // its values [4][S], positions A + 2 B
     // its right-hand side, float4 [T], out of registers while the levels below run on a cluster's CTAs
     static constexpr bool VS = H;
     static constexpr int V1 = E1 + 4 * S;
-    static constexpr int W2 = V1 + (VS ? 4 * T : 0);    // distributed 1/64 (on 1/256): weights, inverse diagonal, values,
+    // distributed 1/64 (on 1/256): weights, inverse diagonal, values
+    static constexpr int W2 = V1 + (VS ? 4 * T : 0);
     static constexpr int ID2 = W2 + (L2 ? 4 * T : 0);
     static constexpr int E2 = ID2 + (L2 ? T : 0);
     static constexpr int RR = E2 + (L2 ? S : 0);   // red residuals of the whole level [2 TOP][2 TOP]
@@ -103,7 +105,7 @@ struct Geo {
     // level below it, whole, in PV; lower ones in D
     static constexpr int KG = PV;
     __host__ __device__ static constexpr int kst(int M) {
-        return M == TOP ? (L2 ? D : PV) : M == 16 ? D + (L2 ? 2 * TOP * TOP : 0) : M == 8 ? kst(16) + 512 : kst(16) + 640;
+        return M == TOP ? (L2 ? D : PV) : M == 16 ? D + (L2 ? 2 * TOP * TOP : 0) : kst(16) + (M == 8 ? 512 : 640);
     }
     // float4s of refinement state of one CTA (device memory): r hi, r lo, x hi, x lo and, with DG, d
     static constexpr int REF4 = (DG ? 20 : 16) * T;
@@ -137,7 +139,10 @@ __device__ __forceinline__ void st_peer(float4* p, int rank, float4 v) {
 }
 __device__ __forceinline__ float2 ld_peer2(const float2* p, int rank) {
     float2 v;
-    asm volatile("ld.shared::cluster.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "r"(peer_addr(p, rank)) : "memory");
+    asm volatile("ld.shared::cluster.v2.f32 {%0, %1}, [%2];"
+                 : "=f"(v.x), "=f"(v.y)
+                 : "r"(peer_addr(p, rank))
+                 : "memory");
     return v;
 }
 // barrier of everything that solves one particle: the block, or the cluster (release / acquire, which also
@@ -221,8 +226,8 @@ __device__ __forceinline__ void invert4(const float* k4, float* dinv) {
 }
 
 // ---- levels that a CTA solves as a whole ---------------------------------------------------------
-// Level M as a grid of M columns and M rows (column 0 and row 0: Dirichlet, always 0), node f = M J + I. A thread takes a red and a black node side by side, so that every
-// lane has work in both colours. Neighbours wrap as above.
+// Level M as a grid of M columns and M rows (column 0 and row 0: Dirichlet, always 0), node f = M J + I. A thread takes
+// a red and a black node side by side, so that every lane has work in both colours. Neighbours wrap as above.
 template <int M>
 __device__ __forceinline__ int wrap(int f) {
     return f & (M * M - 1);
@@ -691,7 +696,7 @@ __device__ __forceinline__ void solve_tile(const FemArgs& a, const int item, flo
             if constexpr (G::VS) reinterpret_cast<float4*>(sm + G::V1)[tid] = make_float4(v00, v10, v01, v11);
             // right-hand side of the node (tx, ty) two levels down
             {
-                        const float l10 = E1[S + pL], b01 = E1[2 * S + pB];
+                const float l10 = E1[S + pL], b01 = E1[2 * S + pB];
                 // the weights of the patch below left (tx = 0: any, the node is a Dirichlet node)
                 const float4 wD = tid < TX ? reinterpret_cast<const float4*>(sm + G::WH)[tx > 0 ? tx - 1 : 0]
                                            : W1[T + tid - TX - (tx > 0 ? 1 : 0)];
@@ -1027,7 +1032,7 @@ __global__ void __launch_bounds__(G::T, G::MINB) fem_tile_kernel(FemArgs a, floa
     __shared__ int item_s[2];
     const int rank = G::H ? cluster_rank() : 0;
     float4* ref = ref_scratch + (size_t)blockIdx.x * G::REF4;
-    if constexpr (G::H) sync_all<G::C>();   // every CTA of the cluster runs before the first store into another's memory
+    if constexpr (G::H) sync_all<G::C>();   // every CTA runs before the first store into another's memory
     grid_wait();
     auto take = [&](int k) {
         const int item = atomicAdd(counter, 1);

@@ -294,7 +294,8 @@ umma_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
             const int row = m0 + 32 * warp + lane;
             const bool in = row < M;
             // rows past the end read the last one: a branch here could leave the warp apart at tmem_ld32
-            const float* pre_in = epi.kind == kEpiGeluBackward ? epi.pre_in + (size_t)min(row, M - 1) * epi.ld_pre : nullptr;
+            const float* pre_in =
+                epi.kind == kEpiGeluBackward ? epi.pre_in + (size_t)min(row, M - 1) * epi.ld_pre : nullptr;
 #pragma unroll 1
             for (int c0 = 0; c0 < BN && n0 + c0 < N; c0 += 32) {
                 const int col = n0 + c0;
@@ -322,7 +323,8 @@ umma_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
                 }
                 __nv_bfloat162 h[16];
 #pragma unroll
-                for (int i = 0; i < 16; ++i) h[i] = __nv_bfloat162(__float2bfloat16_rn(v[2 * i]), __float2bfloat16_rn(v[2 * i + 1]));
+                for (int i = 0; i < 16; ++i)
+                    h[i] = __nv_bfloat162(__float2bfloat16_rn(v[2 * i]), __float2bfloat16_rn(v[2 * i + 1]));
                 if (in) {
                     __nv_bfloat16* act = epi.act + (size_t)row * epi.ld_act + col;
                     st_v8(act, reinterpret_cast<const float*>(h));
