@@ -147,8 +147,9 @@ const char* smc_last_error(const smc_handle* h);
 
 /* Forward map and potential on level `level` (0-based, coarse to fine) for n
  * particles: G_l(theta) (Sec. 2.1, Sec. 5) and Phi_l (Eq. phi). Host arrays:
- * theta [n][K] in, G [n][n_obs] out (may be NULL), Phi [n] out. Copies in and
- * out on the handle's stream and waits for it. n may be 0. Returns
+ * theta [n][K] in, G [n][n_obs] out (may be NULL), Phi [n] out. Runs on the
+ * handle's stream and waits for it: up to 256 KiB in and out by way of pinned
+ * memory that the kernels read and write, larger ones with copies. n may be 0. Returns
  * SMC_ENOCONV if any solve reached opts.max_iter without meeting opts.rtol
  * (its Phi is still written). */
 int smc_eval_likelihood(smc_handle* h, int level, int n, const double* theta,

@@ -26,16 +26,16 @@
 // Why this split: with one node per register slot and everything else in shared memory (the form of
 // fem_solve.cu) a node update reads nine words from shared memory, 21 block barriers an iteration; that
 // form (two 512-thread blocks an SM on 1/64) took 1.99 ms for 4000 particles on 1/64 and 0.42 ms on
-// 1/32. Here a patch of 16 nodes reads 8 rim words per half sweep, 17 barriers an iteration, 256 threads
-// of 128 registers, two blocks an SM (1/64) or 64 threads, eight blocks (1/32): 0.77 ms and 0.17 ms. On
+// 1/32. Here a patch of 16 nodes reads 8 rim words per half sweep, 18 barriers an iteration (1/32: 13), 256
+// threads of 128 registers, two blocks an SM (1/64) or 64 threads, eight blocks (1/32): 0.78 ms and 0.18 ms. On
 // 1/128 (8000 particles) one node per slot on two CTAs of 1024 threads took 31.5 ms, this form 13.1 ms; on
-// 1/256 (1001 particles) the fine levels in device memory took 34.2 ms, this form 12.7 ms.
+// 1/256 (1001 particles) the fine levels in device memory took 34.2 ms, this form 13.2 ms.
 // What bounds it is latency: one 1/64 particle alone on an SM takes 0.87 of the time that two take
 // together. A spill is what hurts most: the direction p lives in shared memory and addresses are formed
-// where they are used, so that (but for ten words around the whole levels in the cluster forms) no register is
+// where they are used, so that (but for a dozen words around the whole levels in the cluster forms) no register is
 // spilled in the iteration (1/64: 0.86 ms with a 20-word spill).
-// The flow cell's solve is not in this form: its observations move by 7e-9 with the order of the dot
-// products (a solve in a thousand then stops one iteration earlier or later, a large step there).
+// The flow cell's solve is not in this form, to keep its bits: its observations move by 7e-9 with the order of the
+// dot products (a solve in a thousand then stops one iteration earlier or later, a large step there).
 #include <cuda_runtime.h>
 
 #include <algorithm>

@@ -39,7 +39,7 @@ long long launch_count();
 
 // ---- forward solve (fem_solve.cu) -------------------------------------------------------
 struct FemArgs {
-    int N;                  // cells per side of this level (power of two, 4..64)
+    int N;                  // cells per side of this level (power of two, 4..256)
     int precision;          // SMC_FP64 or SMC_MIXED
     int n;                  // particles
     int K;                  // KL terms
@@ -66,7 +66,7 @@ struct FemArgs {
     unsigned* bad;          // += solves that did not reach rtol, or null (fem_tile_launch only)
 };
 // Returns cudaSuccess or the launch error.
-// T = threads per particle (one of fem_block_sizes; <= 0: the first, the default)
+// T = the block size (one of fem_block_sizes; <= 0: the first)
 cudaError_t fem_eval_launch(const FemArgs& a, cudaStream_t stream, int T = 0);
 std::vector<int> fem_block_sizes(int N, int precision);
 // those of them that are different kernels, the default first: what the autotuner times

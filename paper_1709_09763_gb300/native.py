@@ -421,7 +421,9 @@ class Handle:
         self._check(self._lib.smc_set_block_size(self._h, int(level), int(T)))
 
     def block_size(self, level):
-        """Threads per particle the solves of `level` run with (negative: a compact form)."""
+        """The block size the solves of `level` run with: threads per particle, or the name of a form (1/32 and
+        1/64 of the mixed path: every size is the register-tiled form; 1/128: -1024 on two CTAs, 1024 in device
+        memory)."""
         T = ctypes.c_int()
         self._check(self._lib.smc_block_size(self._h, int(level), ctypes.byref(T)))
         return T.value
